@@ -99,14 +99,14 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     lmap[kz * kLMS + ky] = (short)l;
   }
   // Iteration form with W (float32 path): this launch is released by the eigen kernel after
-  // that kernel's own wait, so the previous iteration's data-consistency kernel and the sparse
-  // step (joined by an event) have completed: their outputs (X_{k-1}, L_{k-1}, S_{k-1}, S_k)
-  // are read before this wait, while the eigendecomposition still runs; W and the control
-  // block after it.
+  // that kernel's own wait, so the previous iteration's data-consistency kernel and what it waited
+  // for have completed: X_{k-1}, L_{k-1} and S_{k-1} are read before this wait, while the
+  // eigendecomposition still runs; W, the control block and S_k after it (the sparse step beside the
+  // eigen kernel is a programmatic predecessor too, which only the wait waits for).
   const bool iter_form = a.W != nullptr || a.Lpre != nullptr;
   const bool early = a.W != nullptr;
   float dz2 = 0.f, z2 = 0.f;   // ||Z_k - Z_{k-1}||^2, ||Z_{k-1}||^2 (this thread's elements)
-  float2 Sk[EPT], Dz[EPT];
+  float2 Sk[EPT], Dz[EPT];   // S_k, Z_{k-1}
   float2* Mp = gbuf;                // group 0's buffer: M_{k-1} = X_{k-1} - S_{k-1}
   float2* Lsh = gbuf + kNZ * kRS;   // group 1's buffer: L_k
   auto prologue_loads = [&]() {
@@ -114,11 +114,11 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     for (int k = 0; k < EPT; ++k) {
       const int e = tid + k * NTH, z = e / kNY, y = e % kNY;
       const long long gi = (long long)z * xy + xoff + y;
-      Sk[k] = a.S[gi];
-      const float2 Sp = a.Sprev[gi];
-      const float2 Zo = cadd(a.Lbuf[gi], Sp);
-      if (a.W) Mp[z * kRS + y] = csub(a.X[gi], Sp);
-      Dz[k] = csub(Sk[k], Zo);
+      // from L2: this SM's L1 may hold older lines of these arrays before the wait
+      const float2 Sp = __ldcg(a.Sprev + gi);
+      const float2 Zo = cadd(__ldcg(a.Lbuf + gi), Sp);
+      if (a.W) Mp[z * kRS + y] = csub(__ldcg(a.X + gi), Sp);
+      Dz[k] = Zo;
       z2 += cabs2(Zo);
     }
   };
@@ -142,6 +142,11 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
   // ---- prologue: Z = L_k + S_k of the plane into zs -------------------------------------
   if (iter_form) {
     if (!early) prologue_loads();
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+      const int e = tid + k * NTH, z = e / kNY, y = e % kNY;
+      Sk[k] = a.S[(long long)z * xy + xoff + y];
+    }
     if (a.W) {
       for (int i = tid; i < kNZ * kNZ; i += NTH) wsh[i] = a.W[i];
       __syncthreads();
@@ -170,7 +175,7 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
       const long long gi = (long long)z * xy + xoff + y;
       const float2 Lk = a.W ? Lsh[z * kRS + y] : a.Lpre[gi];
       a.Lbuf[gi] = Lk;
-      dz2 += cabs2(cadd(Lk, Dz[k]));
+      dz2 += cabs2(cadd(Lk, csub(Sk[k], Dz[k])));
       zs[z * kRS + y] = cadd(Lk, Sk[k]);   // Z
     }
   } else {
