@@ -20,9 +20,18 @@
 // lambda_S = rel_S max|T(X_0)|.
 #include "lps_internal.cuh"
 
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
+
 namespace lps {
 
 constexpr int kEigThreads = 512;
+// CTAs of the cluster that sums the Gram partials where there are more bytes of them than one SM
+// reads in about a microsecond (160 partials of 24 x 24: 0.74 MB). The first goes on alone. Without
+// it one SM read them in 10 us of the kernel's 48.6 (160 x 160 x 24).
+constexpr int kEigCluster = 8;
+constexpr size_t kEigClusterBytes = 96 * 1024;
 constexpr int kLd = kMaxNc + 1;   // leading dimension of the shared matrices
 
 __device__ __forceinline__ float2 mkc(float x, float y) { return make_float2(x, y); }
@@ -293,7 +302,46 @@ __device__ __forceinline__ float2 gram_chunk(const float2* __restrict__ gram_par
 
 // NCT: the column count fixed at compile time (its loops unroll and their loads pipeline);
 // 0 takes it from the geometry at run time.
-template <int NCT>
+// CTA `rank`'s share of the Gram: ne entries, each summed over the partials in 512 / ne interleaved
+// chunks (a warp reads consecutive entries of a partial), the chunks added in order. Every partial
+// holds an exactly Hermitian matrix and every entry is summed in the same order, so the result is
+// Hermitian too. Ends with the cluster's meeting, after which the first CTA has all of G.
+template <int CL>
+__device__ __forceinline__ void gram_share(const EigArgs& a, EigShared& sh, int nn, int n, int rank,
+                                           cg::cluster_group cl) {
+  const int ne = (nn + CL - 1) / CL, ksub = kEigThreads / ne, e0 = rank * ne;
+  const int tid = threadIdx.x, chunk = tid / ne, idx = tid - chunk * ne;
+  float2* sub = sh.A0;
+  if (chunk < ksub && e0 + idx < nn) {
+    const float2* src = a.gram_part + e0 + idx;
+    constexpr int U = 8;
+    float2 s = make_float2(0.f, 0.f);
+    for (int p0 = chunk; p0 < a.nparts; p0 += ksub * U) {
+      float2 v[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int p = p0 + q * ksub;
+        v[q] = p < a.nparts ? src[(long long)p * nn] : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) s = cadd(s, v[q]);
+    }
+    sub[tid] = s;
+  }
+  __syncthreads();
+  if (tid < ne && e0 + tid < nn) {
+    float2 s = sub[tid];
+    for (int q = 1; q < ksub; ++q) s = cadd(s, sub[q * ne + tid]);
+    const int e = e0 + tid, i = e / n, j = e - i * n;
+    if (i == j) s.y = 0.f;
+    cl.map_shared_rank(sh.G, 0)[i * kLd + j] = s;
+  }
+  cl.sync();
+}
+
+// CL: cluster size. CTA r of a cluster sums the entries [r ne, (r + 1) ne) of the Gram, and stores them
+// in the first CTA's shared memory.
+template <int NCT, int CL>
 __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EigShared& sh = *reinterpret_cast<EigShared*>(smem_raw);
@@ -307,6 +355,15 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   pdl_wait();   // the Gram partials, statistics and control block come from earlier kernels
   pdl_trigger();
   const int nn = n * n;
+  if constexpr (CL > 1) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
+    if (rank > 0) {
+      if (ctrl->converged) return;   // set by this launch only after the cluster has met
+      gram_share<CL>(a, sh, nn, n, rank, cl);
+      return;
+    }
+  }
   const int nut = n * (n + 1) / 2;
   const bool tol_on = a.tol > 0.0;
   // Every independent global load of the kernel is issued before the first barrier: control
@@ -381,7 +438,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   float2* sub = sh.A0;   // scratch [ksub][nn], spans A0 and A1 (free until the Jacobi)
   // at most two tasks per thread: ksub * nn <= 2 * kEigThreads (n <= 32)
   float2 gacc0 = make_float2(0.f, 0.f), gacc1 = make_float2(0.f, 0.f);
-  if (!a.finalize && a.part != 2) {
+  if (CL == 1 && !a.finalize && a.part != 2) {
     gacc0 = gram_chunk(a.gram_part, tid, nn, ksub, a.nparts);
     if (tid + kEigThreads < ksub * nn) gacc1 = gram_chunk(a.gram_part, tid + kEigThreads, nn, ksub, a.nparts);
   }
@@ -394,6 +451,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   }
   __syncthreads();
   if (sh.flags[2]) return;
+  if constexpr (CL > 1) gram_share<CL>(a, sh, nn, n, 0, cg::this_cluster());
 
   // 1. statistics record and the stopping rule (the second part of the float64 mode has done it)
   if (stats_on && (tid >> 5) == sw) {
@@ -434,8 +492,8 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   float2* Vres = sh.V;   // eigenvectors (columns)
   if (a.part != 2) {
     // 2. Gram matrix: combine the chunk sums in a fixed order; exact Hermitian symmetry
-    if (tid < ksub * nn) sub[tid] = gacc0;
-    if (tid + kEigThreads < ksub * nn) sub[tid + kEigThreads] = gacc1;
+    if (CL == 1 && tid < ksub * nn) sub[tid] = gacc0;
+    if (CL == 1 && tid + kEigThreads < ksub * nn) sub[tid + kEigThreads] = gacc1;
     const bool warm = sh.v_valid != 0;
     if (!warm)
       for (int e = tid; e < nn; e += kEigThreads) {
@@ -447,14 +505,16 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
       if (i >= n || j >= n) sh.V[i * kLd + j] = (i == j) ? make_float2(1.f, 0.f) : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    for (int e = tid; e < nn; e += kEigThreads) {
-      const int i = e / n, j = e - i * n;
-      float2 s = sub[e];
-      for (int q = 1; q < ksub; ++q) s = cadd(s, sub[q * nn + e]);
-      if (i == j) s.y = 0.f;
-      sh.G[i * kLd + j] = s;
+    if constexpr (CL == 1) {
+      for (int e = tid; e < nn; e += kEigThreads) {
+        const int i = e / n, j = e - i * n;
+        float2 s = sub[e];
+        for (int q = 1; q < ksub; ++q) s = cadd(s, sub[q * nn + e]);
+        if (i == j) s.y = 0.f;
+        sh.G[i * kLd + j] = s;
+      }
+      __syncthreads();
     }
-    __syncthreads();
 
     // 3. Jacobi, warm-started from the previous eigenvectors
     if (warm) {
@@ -644,17 +704,43 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
 
 
 
-template <int NCT>
-static cudaError_t launch_eig_n(const EigArgs& a, cudaStream_t st) {
+template <int NCT, int CL>
+static cudaError_t launch_eig_c(const EigArgs& a, cudaStream_t st) {
   const size_t smem = sizeof(EigShared);
   static bool attr_set = false;
   if (smem > 48 * 1024 && !attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_eig<NCT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_eig<NCT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  cudaError_t e = launch_pdl(k_eig<NCT>, dim3(1), dim3(kEigThreads), smem, st, a);
+  cudaError_t e;
+  if constexpr (CL == 1) {
+    e = launch_pdl(k_eig<NCT, 1>, dim3(1), dim3(kEigThreads), smem, st, a);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CL);
+    cfg.blockDim = dim3(kEigThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CL;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, k_eig<NCT, CL>, a);
+  }
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int NCT>
+static cudaError_t launch_eig_n(const EigArgs& a, cudaStream_t st) {
+  const size_t bytes = (size_t)a.nparts * a.g.nc * a.g.nc * sizeof(float2);
+  if (!a.finalize && a.part != 2 && bytes > kEigClusterBytes) return launch_eig_c<NCT, kEigCluster>(a, st);
+  return launch_eig_c<NCT, 1>(a, st);
 }
 
 cudaError_t launch_eig(const EigArgs& a, cudaStream_t st) {
