@@ -26,6 +26,12 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-diag-suppres
          f"-I{INCLUDE}", f"-I{CSRC}"]
 
 
+# The factored-row kernel calls its row and column transforms across translation units, under one
+# register limit (so that their largest does not set the kernel's occupancy).
+RDC = ("k_dc_rows.cu", "dc_row_fn", "dc_col_fn")
+RDC_FLAGS = ["-rdc=true", "-maxrregcount=128"]
+
+
 def nvcc() -> str:
     for cand in (os.environ.get("NVCC"), shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
         if cand and os.path.exists(cand):
@@ -52,7 +58,8 @@ def up_to_date() -> bool:
 
 def _compile(src: str) -> str:
     obj = os.path.join(OUT_DIR, os.path.basename(src) + ".o")
-    cmd = [nvcc(), *ARCH, *FLAGS, "-c", src, "-o", obj]
+    rdc = RDC_FLAGS if os.path.basename(src).startswith(RDC) else []
+    cmd = [nvcc(), *ARCH, *FLAGS, *rdc, "-c", src, "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")

@@ -1,9 +1,9 @@
 // Discrete Fourier transforms of compile-time length held in registers (float2 arrays),
-// mixed radix 2, 3, 4, 5, 7, unnormalised:
+// mixed radix 2, 3, 4 and odd primes, unnormalised:
 //   forward  X[k] = sum_n x[n] exp(-2 pi i n k / N),   inverse  with exp(+2 pi i n k / N).
 // Composite lengths split N = P M by decimation in time (P sub-sequences x[P m + r] of length
-// M, twiddles exp(-+2 pi i r k / N), then P-point transforms across r); primes 3, 5, 7 use
-// the symmetric form that pairs x[j] with x[N - j]. The roots are compile-time constants:
+// M, twiddles exp(-+2 pi i r k / N), then P-point transforms across r); odd primes use the
+// symmetric form that pairs x[j] with x[N - j]. The roots are compile-time constants:
 // cos and sin of 2 pi j / N evaluated by Taylor series in double precision and rounded to
 // float when the table is built (constexpr), so no trigonometric call runs on the device.
 // Usable from host code as well (the same template compiles for the CPU), which is how the
@@ -94,8 +94,34 @@ DFT_HD float2 f2(float x, float y) {
   r.y = y;
   return r;
 }
+// Sums, differences and t + s a as one packed instruction on the device (f32x2: each half rounds
+// as the scalar instruction does). The pipe does as many float32 operations either way (126
+// against 124 per clock and SM, measured), but the packed form takes half the issue slots, which
+// is what the transforms run out of.
+#ifdef __CUDA_ARCH__
+#define DFT_PACKED2(OP)                                                                                          \
+  float2 r;                                                                                                      \
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n " OP ".rn.f32x2 z, x, y;\n"         \
+      " mov.b64 {%0, %1}, z;\n}\n"                                                                               \
+      : "=f"(r.x), "=f"(r.y)                                                                                     \
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                                 \
+  return r;
+__device__ __forceinline__ float2 add(float2 a, float2 b) { DFT_PACKED2("add") }
+__device__ __forceinline__ float2 sub(float2 a, float2 b) { DFT_PACKED2("sub") }
+__device__ __forceinline__ float2 axpy(float2 a, float s, float2 t) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z, w;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %4};\n mov.b64 z, {%5, %6};\n"
+      " fma.rn.f32x2 w, x, y, z;\n mov.b64 {%0, %1}, w;\n}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(s), "f"(t.x), "f"(t.y));
+  return r;
+}
+#undef DFT_PACKED2
+#else
 DFT_HD float2 add(float2 a, float2 b) { return f2(a.x + b.x, a.y + b.y); }
 DFT_HD float2 sub(float2 a, float2 b) { return f2(a.x - b.x, a.y - b.y); }
+DFT_HD float2 axpy(float2 a, float s, float2 t) { return f2(t.x + a.x * s, t.y + a.y * s); }
+#endif
 // a * exp(-+2 pi i j / N) for the root j of length N (forward: minus sign)
 template <int N, bool INV>
 DFT_HD float2 rot(float2 a, int j) {
@@ -108,16 +134,20 @@ DFT_HD float2 rot(float2 a, int j) {
   return f2(a.x * c - a.y * s, a.x * s + a.y * c);
 }
 
+// First factor of a composite length: 4 or 2, else the smallest odd prime factor; 0 for a prime.
 template <int N>
 DFT_CX int radix_of() {
-  return (N % 4 == 0 && N > 4) ? 4 : (N % 2 == 0 && N > 2) ? 2 : (N % 3 == 0 && N > 3) ? 3
-                                                            : (N % 5 == 0 && N > 5) ? 5 : (N % 7 == 0 && N > 7) ? 7 : 0;
+  if (N % 4 == 0 && N > 4) return 4;
+  if (N % 2 == 0 && N > 2) return 2;
+  for (int p = 3; p * p <= N; p += 2)
+    if (N % p == 0) return p;
+  return 0;
 }
 
 template <int N, bool INV>
 DFT_HD void dft(float2 (&v)[N]);
 
-// Odd prime N (3, 5, 7): pairs a_j = x_j + x_{N-j}, b_j = x_j - x_{N-j};
+// Odd prime N: pairs a_j = x_j + x_{N-j}, b_j = x_j - x_{N-j};
 // X[k] = x_0 + sum_j a_j cos(2 pi j k / N) -+ i sum_j b_j sin(2 pi j k / N), X[N-k] with +-.
 template <int N, bool INV>
 DFT_HD void dft_prime(float2 (&v)[N]) {
@@ -140,10 +170,8 @@ DFT_HD void dft_prime(float2 (&v)[N]) {
 #pragma unroll
     for (int j = 1; j <= H; ++j) {
       const int q = (j * k) % N;
-      t.x += a[j].x * R.c[q];
-      t.y += a[j].y * R.c[q];
-      u.x += b[j].x * R.s[q];
-      u.y += b[j].y * R.s[q];
+      t = axpy(a[j], R.c[q], t);
+      u = axpy(b[j], R.s[q], u);
     }
     // forward: X[k] = t - i u, X[N-k] = t + i u; inverse swaps them
     const float2 mi = f2(t.x + u.y, t.y - u.x);   // t - i u
@@ -173,11 +201,10 @@ DFT_HD void dft(float2 (&v)[N]) {
     v[2] = sub(s02, s13);
     v[1] = INV ? pi : mi;
     v[3] = INV ? mi : pi;
-  } else if constexpr (N == 3 || N == 5 || N == 7) {
+  } else if constexpr (radix_of<N>() == 0) {
     dft_prime<N, INV>(v);
   } else {
     constexpr int P = radix_of<N>();
-    static_assert(P > 0, "length must factor into 2, 3, 5, 7");
     constexpr int M = N / P;
     float2 s[P][M];
 #pragma unroll

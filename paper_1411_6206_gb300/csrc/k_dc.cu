@@ -1,6 +1,5 @@
-// Launchers of the data-consistency kernel k_dc (k_dc.cuh): runtime-sized Stockham variants
-// (instantiated here) and the register-transform update (instantiated per nz in
-// k_dc_rt_nz*.cu).
+// Launchers of the runtime-sized data-consistency kernel k_dc (k_dc.cuh) and the choice among the
+// data-consistency kernels.
 #include "k_dc.cuh"
 
 #include <algorithm>
@@ -45,48 +44,6 @@ static cudaError_t launch_dc_s(const DcArgs& a, cudaStream_t st) {
   return launch_dc_m<MODE, false, false>(a, st);
 }
 
-cudaError_t launch_dc_fixed(const DcArgs& a, int mode, cudaStream_t st);
-
-// Shared memory of the register-transform update: the direct kernel's layout with the W
-// region replaced by the larger of itself and the transform loop's region.
-static size_t dc_rt_smem_bytes(const Geom& g, int dsm_slots) {
-  Geom gd = g;
-  gd.dc_direct = 1;
-  return dc_smem_bytes(gd) - (size_t)g.nz * g.nz * sizeof(float2) + rt_region_bytes(g.nz, g.ny, dsm_slots);
-}
-
-bool dc_rt_geometry(const Geom& g) {
-  const int q = g.ny / 16;
-  if (g.cs != 1 || g.ny % 16 != 0 || q < 4 || q > 10 || dc_has_fixed(g)) return false;
-  switch (g.nz) {
-    case 8: case 10: case 12: case 14: case 16: case 20: case 24: case 28: case 32: return true;
-    default: return false;
-  }
-}
-
-bool dc_rt_applies(const Geom& g) {
-  return g.dc_rt && !g.dc_generic && dc_rt_geometry(g) && dc_rt_smem_bytes(g, 0) <= 227 * 1024;
-}
-
-// cudaErrorNotSupported where the plane has no register-transform instantiation (or the plan
-// keeps half-precision coil maps, which the runtime-sized kernel reads).
-static cudaError_t launch_dc_rt(const DcArgs& a, cudaStream_t st) {
-  if (!dc_rt_applies(a.g) || a.coils_h) return cudaErrorNotSupported;
-  // slots for a coil's samples in shared memory: the line capacity, or what is left of the
-  // 227 KB (a frame with more lines reads them from L2)
-  DcArgs b = a;
-  const size_t fixed = dc_rt_smem_bytes(a.g, 0);
-  b.g.dc_rt_dsm = (int)std::min<size_t>((size_t)a.g.mpad, (227 * 1024 - fixed) / sizeof(float2)) & ~1;
-  const size_t smem = dc_rt_smem_bytes(b.g, b.g.dc_rt_dsm);
-#define LPS_RT_DISPATCH(NZ) \
-  case NZ: return launch_dc_rt_nz<NZ>(b, smem, st);
-  switch (a.g.nz) {
-    LPS_RT_NZ_LIST(LPS_RT_DISPATCH)
-    default: return cudaErrorNotSupported;
-  }
-#undef LPS_RT_DISPATCH
-}
-
 // One persistent launch over a batch's descriptor table (operator form of the update): each CTA
 // takes (member, plane) items from an atomic counter, copies the member's arguments to shared
 // memory and runs the plane with the runtime-sized body (coil maps read from L2, up to 24
@@ -111,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dc_persist(const DcArgs* __rest
     int* dst = reinterpret_cast<int*>(&sa);
     for (int i = threadIdx.x; i < (int)(sizeof(DcArgs) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
     __syncthreads();
-    dc_plane<24, kDcUpdate, false, false, 0, 0>(sa, it - start[m]);
+    dc_plane<24, kDcUpdate, false, false>(sa, it - start[m]);
     __syncthreads();
   }
 }
@@ -149,18 +106,17 @@ cudaError_t launch_dc_persist(const DcArgs* table, const int* start, int nm, int
 }
 
 // The update of a 128 x 16 plane goes to the register-transform kernel (k_dc_reg) unless the
-// plan selected another variant; planes of ny = 16 Q (Q = 4..10) by even nz <= 32 to k_dc with
-// the register-transform coil loop; other plane sizes with a compile-time specialisation go to
-// k_dc_fixed; the rest to k_dc.
+// plan selected another variant; the 32 x 8 plane to k_dc_fixed; planes that factor (dc_rows.cuh) to
+// k_dc_rows; the rest, and plans that selected a runtime-sized variant, to k_dc.
 cudaError_t launch_dc(const DcArgs& a, int mode, cudaStream_t st) {
   if (mode == kDcUpdate) {
     const cudaError_t er = launch_dc_reg(a, st);
     if (er != cudaErrorNotSupported) return er;
-    const cudaError_t et = launch_dc_rt(a, st);
-    if (et != cudaErrorNotSupported) return et;
   }
   const cudaError_t ef = launch_dc_fixed(a, mode, st);
   if (ef != cudaErrorNotSupported) return ef;
+  const cudaError_t ew = launch_dc_rows(a, mode, st);
+  if (ew != cudaErrorNotSupported) return ew;
   if (dc_smem_bytes(a.g) > 227 * 1024) return cudaErrorInvalidValue;
   switch (mode) {
     case kDcUpdate: return launch_dc_s<kDcUpdate>(a, st);

@@ -37,7 +37,7 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
 unsigned char* g_dev_scratch[kMaxDevices] = {};   // device address of the array, per device
-int g_lines[1024 * LPS_MAX_NC];                     // host staging of the line table (static)
+alignas(16) int g_lines[1024 * LPS_MAX_NC];         // host staging of the line table or row tasks (static)
 float2 g_tw[3 * 1024];                              // host staging of the twiddles (static)
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -133,10 +133,20 @@ extern "C" int lps_adjoint_noalloc(int nx, int ny, int nz, int ncoil, int fft_z,
   float2* hyb = reinterpret_cast<float2*>(base + o_hyb);
 
   // host-side tables (static staging buffers, copied before the call returns)
-  int k = 0;
-  for (int a = 0; a < nz; ++a)
-    for (int ky = 0; ky < ny; ++ky)
-      if (mask[(size_t)a * ny + ky]) g_lines[k++] = a * g.nyp + ky;
+  // line table, or, where the plane has a factored-row form and they fit its place, the row tasks and
+  // raster numbers that the kernels of that form read instead (the samples then lie in task order)
+  const size_t task_bytes = dc_rows_geometry(g) && !dc_small_applies(g) ? dc_row_task_bytes(g) : 0;
+  const bool rows = task_bytes > 0 && task_bytes + (size_t)m * sizeof(short) <= (size_t)ny * nz * sizeof(int);
+  size_t line_bytes = (size_t)m * sizeof(int);
+  if (rows) {
+    line_bytes = task_bytes + (size_t)m * sizeof(short);
+    dc_row_tasks(g, mask, g_lines, nullptr, reinterpret_cast<unsigned short*>(reinterpret_cast<unsigned char*>(g_lines) + task_bytes));
+  } else {
+    int k = 0;
+    for (int a = 0; a < nz; ++a)
+      for (int ky = 0; ky < ny; ++ky)
+        if (mask[(size_t)a * ny + ky]) g_lines[k++] = a * g.nyp + ky;
+  }
   auto fill_tw = [](float2* t, int n) {
     for (int q = 0; q < n; ++q) {
       const double ang = 2.0 * M_PI * (double)q / (double)n;
@@ -155,7 +165,7 @@ extern "C" int lps_adjoint_noalloc(int nx, int ny, int nz, int ncoil, int fft_z,
       cudaMemcpyAsync(tw_x, g_tw, (size_t)nx * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(tw_y, g_tw + nx, (size_t)ny * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(tw_z, g_tw + nx + ny, (size_t)nz * sizeof(float2), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(lines, g_lines, (size_t)m * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess) {
+      cudaMemcpyAsync(lines, g_lines, line_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
     set_err("lps_adjoint_noalloc: table upload failed: %s", cudaGetErrorString(cudaGetLastError()));
     return LPS_ERR_CUDA;
   }
@@ -165,6 +175,7 @@ extern "C" int lps_adjoint_noalloc(int nx, int ny, int nz, int ncoil, int fft_z,
   x.in = static_cast<const float2*>(kdata);
   x.out = hyb;
   x.tw_x = tw_x;
+  if (rows) x.raster = reinterpret_cast<const unsigned short*>(reinterpret_cast<unsigned char*>(lines) + task_bytes);
   x.persist = persist;
   x.inverse = 1;
   cudaError_t le = launch_xfft(x, st);
@@ -177,6 +188,7 @@ extern "C" int lps_adjoint_noalloc(int nx, int ny, int nz, int ncoil, int fft_z,
   d.coils = static_cast<const float2*>(coils);
   d.dhyb = hyb;
   d.lines = lines;
+  if (rows) d.tasks = reinterpret_cast<const RowTask*>(lines);
   d.tw_y = tw_y;
   d.tw_z = tw_z;
   d.persist = persist;

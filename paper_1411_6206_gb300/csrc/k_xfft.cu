@@ -30,11 +30,12 @@ __global__ void __launch_bounds__(kThreads) k_xfft(const XfftArgs a) {
   const int tid = threadIdx.x;
   for (int i = tid; i < nx; i += kThreads) tw[i] = a.tw_x[i];
   const int tot = kLines * nx;
+  auto line_of = [&](int l) { return a.raster ? a.raster[l0 + l] : l0 + l; };   // in the user's order
   if (a.inverse) {
-    const float2* src = a.in + ((long long)c * m + l0) * nx;
+    const float2* src = a.in + (long long)c * m * nx;
     for (int e = tid; e < tot; e += kThreads) {
       const int l = e / nx, k = e - (e / nx) * nx;
-      bufA[l * nxp + k] = (l < nl) ? src[(long long)l * nx + k] : make_float2(0.f, 0.f);
+      bufA[l * nxp + k] = (l < nl) ? src[(long long)line_of(l) * nx + k] : make_float2(0.f, 0.f);
     }
   } else {
     for (int e = tid; e < tot; e += kThreads) {
@@ -55,10 +56,10 @@ __global__ void __launch_bounds__(kThreads) k_xfft(const XfftArgs a) {
       if (l < nl) a.out[((long long)xl * g.ncoil + c) * g.mpad + l0 + l] = cscale(s[l * nxp + x0 + xl], sc);
     }
   } else {
-    float2* dst = a.out + ((long long)c * m + l0) * nx;
+    float2* dst = a.out + (long long)c * m * nx;
     for (int e = tid; e < tot; e += kThreads) {
       const int l = e / nx, k = e - (e / nx) * nx;
-      if (l < nl) dst[(long long)l * nx + k] = cscale(s[l * nxp + k], sc);
+      if (l < nl) dst[(long long)line_of(l) * nx + k] = cscale(s[l * nxp + k], sc);
     }
   }
 }

@@ -193,6 +193,12 @@ int gram_parts(const Geom& g, int precision) {
 }
 int gram_part_capacity(const Geom& g) { return std::max(g.nx, gram_tc_parts(g)); }
 
+// Row tasks (where the plane has them), line positions and raster numbers of a mask.
+size_t line_table_bytes(const Geom& g) {
+  const size_t lines = (size_t)g.plane * sizeof(int);
+  return dc_rows_geometry(g) ? dc_row_task_bytes(g) + lines + (size_t)g.plane * sizeof(short) : lines;
+}
+
 size_t arena_size(const Geom& g, int max_iters) {
   auto r = [](size_t b) { return ((b + 255) / 256) * 256; };
   size_t s = 0;
@@ -200,7 +206,7 @@ size_t arena_size(const Geom& g, int max_iters) {
   s += 4 * r((size_t)g.nc * g.nc * sizeof(float2));      // W, V, float64 mode: Gram, refined V
   s += r((size_t)g.nc * g.nc * sizeof(double2)) + r((size_t)g.nc * sizeof(double));   // A, eigenvalues
   s += r((size_t)g.nxt * sizeof(float2)) + r((size_t)g.ny * sizeof(float2)) + r((size_t)g.nz * sizeof(float2));
-  s += r((size_t)g.plane * sizeof(int));                  // line table
+  s += r(line_table_bytes(g));                            // row tasks, line table, raster numbers
   s += r((size_t)g.nx * 4 * sizeof(float)) + 2 * r((size_t)g.ntiles * 2 * sizeof(float));   // statistic partials
   s += 2 * r((size_t)g.nc * sizeof(double));
   s += 3 * r((size_t)(g.N / 32) * sizeof(uint32_t));   // support: prior, output, second output
@@ -296,8 +302,9 @@ int validate(const lps_params* p, Geom* gout) {
   // 128 x 16 planes: the update runs on the register-transform kernel (four coil groups; their
   // sums in shared memory when there are more than four coils)
   if (g.ny == 128 && g.nz == 16) g.dc_reg_groups = g.ncoil > 4 ? 104 : 4;
-  // planes of ny = 16 Q by even nz <= 32: the update's coil loop on register transforms
-  g.dc_rt = dc_rt_geometry(g) ? 1 : 0;
+  g.dc_small = 1;
+  // planes that factor: every mode of the data-consistency kernel on factored rows
+  g.dc_rows = dc_rows_geometry(g) ? 1 : 0;
   if (dc_ept(g) < 0 || dc_smem_bytes(g) > 227 * 1024) {
     set_err("x-plane of %d x %d does not fit one CTA", p->ny, p->nz);
     return LPS_ERR_UNSUPPORTED;
@@ -394,6 +401,7 @@ DcArgs dc_args(lps_plan* P) {
   a.dhyb = P->dhyb;
   a.dhyb_h = P->dhyb_h;
   a.lines = P->lines;
+  a.tasks = P->tasks;
   a.tw_y = P->tw_y;
   a.tw_z = P->tw_z;
   a.persist = P->persist;
@@ -854,7 +862,12 @@ int lps_plan_create(const lps_params* p, void* stream, lps_plan** out) {
   if ((rc = aalloc(P, &P->tw_x, (size_t)g.nxt))) return fail(rc);
   if ((rc = aalloc(P, &P->tw_y, (size_t)g.ny))) return fail(rc);
   if ((rc = aalloc(P, &P->tw_z, (size_t)g.nz))) return fail(rc);
-  if ((rc = aalloc(P, &P->lines, (size_t)g.plane))) return fail(rc);
+  {
+    unsigned char* t;
+    if ((rc = aalloc(P, &t, line_table_bytes(g)))) return fail(rc);
+    if (dc_rows_geometry(g)) P->tasks = reinterpret_cast<RowTask*>(t);
+    P->lines = reinterpret_cast<int*>(t + (P->tasks ? dc_row_task_bytes(g) : 0));
+  }
   if ((rc = aalloc(P, &P->hist, (size_t)p->max_iters + 2))) return fail(rc);
   if ((rc = aalloc(P, &P->gram_part, (size_t)gram_part_capacity(g) * g.nc * g.nc))) return fail(rc);
   if ((rc = aalloc(P, &P->sup_out, support_words(g)))) return fail(rc);
@@ -862,7 +875,7 @@ int lps_plan_create(const lps_params* p, void* stream, lps_plan** out) {
   if ((rc = aalloc(P, &P->sup_prior, support_words(g)))) return fail(rc);
   if (cudaMallocHost((void**)&P->h_ctrl, sizeof(DevCtrl)) != cudaSuccess ||
       cudaMallocHost((void**)&P->h_persist_slots, lps_plan::kSlots * sizeof(DevPersist)) != cudaSuccess ||
-      cudaMallocHost((void**)&P->h_lines_slots, (size_t)lps_plan::kSlots * g.plane * sizeof(int)) != cudaSuccess) {
+      cudaMallocHost((void**)&P->h_lines_slots, (size_t)lps_plan::kSlots * line_table_bytes(g)) != cudaSuccess) {
     set_err("pinned host allocation failed");
     return fail(LPS_ERR_OOM);
   }
@@ -946,12 +959,21 @@ int lps_set_mask(lps_plan* P, const uint8_t* mask, int* nlines) {
   if (rc) return rc;
   int slot;
   if ((rc = acquire_slot(P, &slot))) return rc;
-  int* hl = P->h_lines_slots + (size_t)slot * P->g.plane;
-  int k = 0;
-  for (int a = 0; a < nz; ++a)
-    for (int ky = 0; ky < ny; ++ky)
-      if (h[(size_t)a * ny + ky]) hl[k++] = a * P->g.nyp + ky;
-  CK(cudaMemcpyAsync(P->lines, hl, (size_t)m * sizeof(int), cudaMemcpyHostToDevice, P->st));
+  unsigned char* hs = P->h_lines_slots + (size_t)slot * line_table_bytes(P->g);
+  if (P->tasks) {
+    const size_t tb = dc_row_task_bytes(P->g);
+    int* hl = reinterpret_cast<int*>(hs + tb);
+    dc_row_tasks(P->g, h, hs, hl, reinterpret_cast<unsigned short*>(hl + m));
+    P->raster = reinterpret_cast<unsigned short*>(P->lines + m);
+    CK(cudaMemcpyAsync(P->tasks, hs, tb + (size_t)m * (sizeof(int) + sizeof(short)), cudaMemcpyHostToDevice, P->st));
+  } else {
+    int* hl = reinterpret_cast<int*>(hs);
+    int k = 0;
+    for (int a = 0; a < nz; ++a)
+      for (int ky = 0; ky < ny; ++ky)
+        if (h[(size_t)a * ny + ky]) hl[k++] = a * P->g.nyp + ky;
+    CK(cudaMemcpyAsync(P->lines, hl, (size_t)m * sizeof(int), cudaMemcpyHostToDevice, P->st));
+  }
   P->nlines = m;
   P->hp.nlines = m;
   if ((rc = upload_persist(P, false, slot))) return rc;
@@ -980,6 +1002,7 @@ int lps_set_data(lps_plan* P, const void* kdata, int nlines) {
   a.in = (const float2*)src;
   a.out = P->dhyb;
   a.tw_x = P->tw_x;
+  a.raster = P->raster;
   a.persist = P->persist;
   a.inverse = 1;
   LK(launch_xfft(a, P->st));
@@ -1248,6 +1271,7 @@ int lps_forward(lps_plan* P, const void* image, void* kdata) {
   x.in = P->hscratch;
   x.out = dev ? (float2*)kdata : P->kstage;
   x.tw_x = P->tw_x;
+  x.raster = P->raster;
   x.persist = P->persist;
   x.inverse = 0;
   LK(launch_xfft(x, P->st));
@@ -1276,6 +1300,7 @@ int lps_adjoint(lps_plan* P, const void* kdata, void* image) {
   x.in = src;
   x.out = P->hscratch;
   x.tw_x = P->tw_x;
+  x.raster = P->raster;
   x.persist = P->persist;
   x.inverse = 1;
   LK(launch_xfft(x, P->st));

@@ -62,6 +62,8 @@ inline double iter_objective(const IterRec& r, float lambda_L, float lambda_S) {
   return 0.5 * (double)r.resid2 + (double)lambda_L * r.nuclear + (double)lambda_S * (double)r.l1;
 }
 
+struct RowTask;   // dc_rows.cuh
+
 struct Geom {
   int nx, ny, nz, ncoil;    // nx: the x-planes this plan holds (a slab of nxt planes)
   int nxt, x0;              // x extent of the whole volume (readout length) and the slab's first plane
@@ -84,8 +86,8 @@ struct Geom {
   int dc_direct;            // runtime-sized kernel reads coil maps from global memory (no staging)
   int lrs_tpc;              // 8x8 tiles per CTA of the sparse-step kernel (0: 32 / nc)
   int dc_reg_groups;        // register-transform DC kernel (128 x 16 planes): coil groups, 0 = off
-  int dc_rt;                // update on k_dc's register-transform coil loop where the plane has one
-  int dc_rt_dsm;            // that loop's shared-memory slots for a coil's samples (set at launch)
+  int dc_small;             // the 32 x 8 plane's own kernel (k_dc_fixed)
+  int dc_rows;              // factored-row kernel (k_dc_rows) where the plane has one
 };
 
 // ---- data-consistency / adjoint / forward kernel (one CTA per x-plane) -------------
@@ -114,6 +116,7 @@ struct DcArgs {
   const float2* dhyb;       // [nx][ncoil][mpad] hybrid-space samples
   float2* hyb_out;          // forward: [nx][ncoil][mpad]
   const int* lines;         // padded in-plane position kz*nyp + ky of each line
+  const RowTask* tasks;     // row tasks of the mask for k_dc_rows (dc_rows.cuh); nullptr = not used
   const float2* tw_y;
   const float2* tw_z;
   float2* gram_part;        // [nx][nc][nc]; nullptr = skip
@@ -128,6 +131,7 @@ struct XfftArgs {
   const float2* in;
   float2* out;
   const float2* tw_x;
+  const unsigned short* raster;   // the user's number of each line; nullptr: the plan's order is the user's
   const DevPersist* persist;
   int inverse;              // 1: k-space [c][l][kx] -> hybrid [x][c][l] (the plan's planes x0 .. x0+nx-1);
                             // 0: the reverse (planes outside the slab count as zero)
@@ -222,8 +226,13 @@ int lrs_tpc(const Geom& g);
 int lrs_threads(const Geom& g);
 bool dc_has_fixed(const Geom& g);
 bool dc_reg_applies(const Geom& g);
-bool dc_rt_geometry(const Geom& g);   // a register-transform instantiation exists for the plane
-bool dc_rt_applies(const Geom& g);
+bool dc_small_applies(const Geom& g);
+cudaError_t launch_dc_fixed(const DcArgs& a, int mode, cudaStream_t st);
+bool dc_rows_geometry(const Geom& g);   // the plane has a factored-row form
+bool dc_rows_applies(const Geom& g);
+size_t dc_row_task_bytes(const Geom& g);
+void dc_row_tasks(const Geom& g, const unsigned char* mask, void* tasks, int* lines, unsigned short* raster);   // host
+cudaError_t launch_dc_rows(const DcArgs& a, int mode, cudaStream_t st);
 // persistent batch form of the update (operator form): one launch over a descriptor table
 bool dc_persist_fits(const Geom& g);
 size_t dc_persist_smem(const Geom& g);
