@@ -317,51 +317,6 @@ __global__ void __launch_bounds__(1024) k_lrs(const LrsArgs a) {
   if (tid == 0) part[1] = r;
 }
 
-// Partials of the Casorati Gram (X - S)^H (X - S) straight from global memory; used when
-// the state is loaded from outside rather than produced by the data-consistency step. CTA p
-// sums the planes x = p q .. p q + q - 1 (q = nx / nparts), so the eigen kernel finds the
-// same number of partials as the data-consistency step leaves.
-__global__ void __launch_bounds__(kThreads) k_gram_plane(const float2* X, const float2* S, Geom g,
-                                                         float2* gram_part, int nparts) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float2* M = reinterpret_cast<float2*>(smem);   // [nz][nyp]
-  const int ny = g.ny, nyp = g.nyp, nc = g.nc;
-  const int q = g.nx / nparts;
-  const long long nxy = (long long)g.nx * ny;
-  float2* gp = gram_part + (long long)blockIdx.x * nc * nc;
-  for (int x = blockIdx.x * q; x < (int)(blockIdx.x + 1) * q; ++x) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < g.plane; e += kThreads) {
-      const int z = e / ny, y = e - (e / ny) * ny;
-      const long long gi = z * nxy + (long long)x * ny + y;
-      M[z * nyp + y] = S ? csub(X[gi], S[gi]) : X[gi];
-    }
-    __syncthreads();
-    const bool first = x == (int)blockIdx.x * q;
-    // each thread owns its entries across the planes, so the running sums need no barrier;
-    // column i holds slices i cs .. i cs + cs - 1
-    for (int t = threadIdx.x; t < nc * nc; t += kThreads) {
-      const int i = t / nc, j = t - (t / nc) * nc;
-      if (i > j) continue;
-      float sr = 0.f, si = 0.f;
-      for (int s = 0; s < g.cs; ++s)
-        for (int y = 0; y < ny; ++y) {
-          const float2 u = M[(i * g.cs + s) * nyp + y], v = M[(j * g.cs + s) * nyp + y];
-          sr = fmaf(u.x, v.x, fmaf(u.y, v.y, sr));
-          si = fmaf(u.x, v.y, fmaf(-u.y, v.x, si));
-        }
-      if (!first) {
-        const float2 o = gp[i * nc + j];
-        sr += o.x;
-        si += o.y;
-      }
-      if (i == j) si = 0.f;   // exactly real diagonal
-      gp[i * nc + j] = make_float2(sr, si);
-      if (i != j) gp[j * nc + i] = make_float2(sr, -si);
-    }
-  }
-}
-
 // recon = L + S, the reconstructed volume of Algorithm 1's output.
 __global__ void k_combine(const float2* __restrict__ L, const float2* __restrict__ S, float2* __restrict__ out,
                           long long n) {
@@ -449,68 +404,6 @@ cudaError_t launch_settle(const DevCtrl* ctrl, int k0, float2* S0, const float2*
                           cudaStream_t st) {
   const int blocks = (int)std::min<long long>((n + 255) / 256, 152LL * 4);
   k_settle<<<blocks, 256, 0, st>>>(ctrl, k0, S0, S1, n, sup0, sup1, nw, part0, part1, np);
-  return cudaGetLastError();
-}
-
-// G = sum of the nparts partials, in partial order (one thread per entry).
-__global__ void k_gram_sum(const float2* __restrict__ part, int nparts, int nn, float2* __restrict__ G) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nn) return;
-  float2 s = make_float2(0.f, 0.f);
-  for (int p = 0; p < nparts; ++p) s = cadd(s, part[(long long)p * nn + e]);
-  G[e] = s;
-}
-
-cudaError_t launch_gram_sum(const float2* part, int nparts, int nc, float2* G, cudaStream_t st) {
-  const int nn = nc * nc;
-  k_gram_sum<<<(nn + 255) / 256, 256, 0, st>>>(part, nparts, nn, G);
-  return cudaGetLastError();
-}
-
-// L[j][r] = sum_i (X - S)[i][r] W[i][j] in float32, one thread per pixel r (the stand-alone
-// form of the reprojection that k_lrs fuses with the sparse step).
-__global__ void k_reproj_f32(const float2* __restrict__ X, const float2* __restrict__ S,
-                             const float2* __restrict__ W, float2* __restrict__ L, Geom g) {
-  const long long nr = g.N / g.nc;   // rows of the Casorati matrix (voxels of a column)
-  const int nc = g.nc;
-  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < nr; r += (long long)gridDim.x * blockDim.x) {
-    float2 m[kMaxNc];
-#pragma unroll
-    for (int i = 0; i < kMaxNc; ++i)
-      m[i] = i < nc ? (S ? csub(X[i * nr + r], S[i * nr + r]) : X[i * nr + r]) : make_float2(0.f, 0.f);
-    for (int j = 0; j < nc; ++j) {
-      float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < kMaxNc; ++i) {
-        if (i < nc) {
-          const float2 w = W[i * nc + j];
-          acc.x = fmaf(m[i].x, w.x, fmaf(-m[i].y, w.y, acc.x));
-          acc.y = fmaf(m[i].x, w.y, fmaf(m[i].y, w.x, acc.y));
-        }
-      }
-      L[j * nr + r] = acc;
-    }
-  }
-}
-
-cudaError_t launch_reproj_f32(const float2* X, const float2* S, const float2* W, float2* L, const Geom& g,
-                              cudaStream_t st) {
-  const long long nr = g.N / g.nc;
-  const int blocks = (int)std::min<long long>((nr + 127) / 128, 152LL * 8);
-  k_reproj_f32<<<blocks, 128, 0, st>>>(X, S, W, L, g);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gram_plane(const float2* X, const float2* S, const Geom& g, float2* gram_part, int nparts,
-                              cudaStream_t st) {
-  if (nparts <= 0 || g.nx % nparts != 0) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)g.planeP * sizeof(float2);
-  if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_gram_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k_gram_plane<<<nparts, kThreads, smem, st>>>(X, S, g, gram_part, nparts);
   return cudaGetLastError();
 }
 

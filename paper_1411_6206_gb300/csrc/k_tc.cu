@@ -28,7 +28,8 @@ namespace lps {
 
 namespace {
 
-constexpr int kTcThreads = 128;       // thread t owns pixel t of a tile and tensor-memory lane t
+constexpr int kTcThreads = 128;       // reprojection: thread t owns pixel t of a tile and tensor-memory lane t
+constexpr int kGramTcThreads = 256;   // Gram: a thread splits 8 pixels of a column at a time
 constexpr int kTcTile = 128;          // pixels per tile
 constexpr uint32_t kTmemCols = 64;    // accumulator columns (N <= 64)
 
@@ -36,6 +37,11 @@ struct Bf16Op {
   using T = uint16_t;
   static constexpr int kBytes = 2;
   static constexpr uint32_t kFmt = 1;   // instruction-descriptor format code (kind::f16, BF16)
+  // a 16-byte core-matrix row
+  __device__ static __forceinline__ uint4 pack(const T (&v)[8]) {
+    return make_uint4(v[0] | (uint32_t)v[1] << 16, v[2] | (uint32_t)v[3] << 16, v[4] | (uint32_t)v[5] << 16,
+                      v[6] | (uint32_t)v[7] << 16);
+  }
   __device__ static __forceinline__ void split(float x, T& hi, T& lo) {
     const __nv_bfloat16 h = __float2bfloat16_rn(x);
     const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
@@ -48,6 +54,7 @@ struct Tf32Op {
   using T = uint32_t;
   static constexpr int kBytes = 4;
   static constexpr uint32_t kFmt = 2;   // kind::tf32
+  __device__ static __forceinline__ uint4 pack(const T (&v)[4]) { return make_uint4(v[0], v[1], v[2], v[3]); }
   __device__ static __forceinline__ void split(float x, T& hi, T& lo) {
     uint32_t h, l;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
@@ -137,6 +144,18 @@ __device__ __forceinline__ void st_op(unsigned char* base, uint32_t off, typenam
   *reinterpret_cast<typename Op::T*>(base + off) = v;
 }
 
+// Consecutive complex values, two to a float4; by 16-byte loads where the address allows.
+template <int C>
+__device__ __forceinline__ void load_row(const float2* p, bool wide, float4 (&v)[C]) {
+  if (wide) {
+#pragma unroll
+    for (int i = 0; i < C; ++i) v[i] = reinterpret_cast<const float4*>(p)[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < C; ++i) v[i] = make_float4(p[2 * i].x, p[2 * i].y, p[2 * i + 1].x, p[2 * i + 1].y);
+  }
+}
+
 __device__ __forceinline__ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 }  // namespace
@@ -144,9 +163,13 @@ __device__ __forceinline__ int round_up(int v, int m) { return (v + m - 1) / m *
 // ---- Gram: G_p = sum over this CTA's tiles of M^H M -------------------------------------
 // A = [Qh^T; Ql^T] (4n rows, zero-padded to 128) times B = Qh (the first N rows of the same
 // buffer) gives D = [Qh^T Qh; Ql^T Qh]; G_real = D_top + D_bot + D_bot^T. Two stages of
-// kTcTile pixels: threads fill one while the tensor core reads the other.
+// kTcTile pixels: threads fill one while the tensor core reads the other. A task is one column and the
+// pixels of one core-matrix row (8 or 4 consecutive pixels): 16-byte loads, and one 16-byte store for
+// each of Re hi, Im hi, Re lo, Im lo. Up to three CTAs share an SM (one with tf32 operands), so
+// that one's loads and splits pass while another waits. Bound by the latency of the loads of the one or two tiles a CTA
+// gets (19 MB in 14 us at 192 x 192 x 32; 19 us with a pixel a thread, 2-byte stores and one CTA an SM).
 template <class Op>
-__global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
+__global__ void __launch_bounds__(kGramTcThreads) k_gram_tc(const GramTcArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int CE = 16 / Op::kBytes;
   constexpr int KC = kTcTile / CE;               // K chunks per stage
@@ -155,7 +178,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
   unsigned char* stage[2] = {smem, smem + SB};
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * SB);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
-  int* flag = reinterpret_cast<int*>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = a.g.nc;
   const int N = round_up(2 * n, 16);
@@ -168,10 +190,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     fence_mbar_init();
-    *flag = 0;
   }
-  for (uint32_t i = tid * 16; i < 2 * SB; i += kTcThreads * 16)
-    *reinterpret_cast<uint4*>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
+  // rows past the 4n that the tiles write: zero (whole row groups from the first partial one)
+  for (uint32_t i = (uint32_t)(4 * n / 8) * KC * 128u + tid * 16; i < SB; i += kGramTcThreads * 16) {
+    *reinterpret_cast<uint4*>(stage[0] + i) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(stage[1] + i) = make_uint4(0u, 0u, 0u, 0u);
+  }
   pdl_trigger();
   pdl_wait();   // X and S come from the preceding kernels
   fence_proxy_async();
@@ -181,6 +205,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
   const uint32_t tmem = *tslot;
   const uint32_t idesc = instr_desc(Op::kFmt, 128, N);
   const int conv = a.ctrl ? a.ctrl->converged : 0;
+  // the caller's images may start on an odd complex value
+  const bool wide = ((reinterpret_cast<uintptr_t>(a.X) | reinterpret_cast<uintptr_t>(a.S)) & 15) == 0;
 
   int it = 0;
   bool bad = false;
@@ -192,28 +218,38 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
       bad = true;
       break;
     }
-    const long long r = (long long)tile * kTcTile + tid;
-    float2 m[kMaxNc];
-#pragma unroll
-    for (int z = 0; z < kMaxNc; ++z) {
-      m[z] = make_float2(0.f, 0.f);
-      if (z < n && r < nr) {
-        const float2 x = a.X[z * nr + r];
-        m[z] = a.S ? csub(x, a.S[z * nr + r]) : x;
-      }
-    }
     unsigned char* st = stage[s];
+    // a column of nx ny pixels is a multiple of 64: a core-matrix row lies inside it or past its end
+#pragma unroll 2
+    for (int t = tid; t < n * KC; t += kGramTcThreads) {
+      const int z = t / KC, c = t - z * KC;
+      const long long r = (long long)tile * kTcTile + c * CE;
+      float2 m[CE];
+      if (r < nr) {
+        float4 x4[CE / 2], s4[CE / 2];
+        load_row(a.X + z * nr + r, wide, x4);
 #pragma unroll
-    for (int z = 0; z < kMaxNc; ++z) {
-      if (z < n) {
-        typename Op::T rh, rl, ih, il;
-        Op::split(m[z].x, rh, rl);
-        Op::split(m[z].y, ih, il);
-        st_op<Op>(st, core_off<Op>(z, tid, KC), rh);
-        st_op<Op>(st, core_off<Op>(n + z, tid, KC), ih);
-        st_op<Op>(st, core_off<Op>(2 * n + z, tid, KC), rl);
-        st_op<Op>(st, core_off<Op>(3 * n + z, tid, KC), il);
+        for (int i = 0; i < CE / 2; ++i) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a.S) load_row(a.S + z * nr + r, wide, s4);
+#pragma unroll
+        for (int i = 0; i < CE / 2; ++i) {
+          m[2 * i] = make_float2(x4[i].x - s4[i].x, x4[i].y - s4[i].y);
+          m[2 * i + 1] = make_float2(x4[i].z - s4[i].z, x4[i].w - s4[i].w);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < CE; ++i) m[i] = make_float2(0.f, 0.f);
       }
+      typename Op::T rh[CE], rl[CE], ih[CE], il[CE];
+#pragma unroll
+      for (int i = 0; i < CE; ++i) {
+        Op::split(m[i].x, rh[i], rl[i]);
+        Op::split(m[i].y, ih[i], il[i]);
+      }
+      *reinterpret_cast<uint4*>(st + core_off<Op>(z, c * CE, KC)) = Op::pack(rh);
+      *reinterpret_cast<uint4*>(st + core_off<Op>(n + z, c * CE, KC)) = Op::pack(ih);
+      *reinterpret_cast<uint4*>(st + core_off<Op>(2 * n + z, c * CE, KC)) = Op::pack(rl);
+      *reinterpret_cast<uint4*>(st + core_off<Op>(3 * n + z, c * CE, KC)) = Op::pack(il);
     }
     fence_proxy_async();
     __syncthreads();
@@ -239,7 +275,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
   // epilogue: D rows -> shared memory (stage 0 is free now), then this CTA's partial
   float* Dsh = reinterpret_cast<float*>(smem);   // [128][N + 1]
   const int ldd = N + 1;
-  if (!bad && it > 0) {
+  if (!bad && it > 0 && warp < 4) {   // warps 0..3 hold the tensor-memory lanes
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
     for (int c0 = 0; c0 < N; c0 += 16) {
       float v[16];
@@ -259,7 +295,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
   auto greal = [&](int p, int q) {   // (Qh^T Qh + Ql^T Qh + Qh^T Ql)[p][q]
     return Dsh[p * ldd + q] + Dsh[(2 * n + p) * ldd + q] + Dsh[(2 * n + q) * ldd + p];
   };
-  for (int e = tid; e < n * n; e += kTcThreads) {
+  for (int e = tid; e < n * n; e += kGramTcThreads) {
     const int i = e / n, j = e - (e / n) * n;
     if (i > j) continue;
     float2 v = make_float2(0.f, 0.f);
@@ -273,16 +309,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gram_tc(const GramTcArgs a) {
 }
 
 // ---- reprojection: L = M W for 128-pixel tiles ------------------------------------------
-// A = [Mh | Mh | Ml] (128 pixels x 6n), B = [Wh; Wl; Wh] (6n x 2n): D = Mh Wh + Mh Wl + Ml Wh.
+// D = Mh Wh + Mh Wl + Ml Wh with A = [Mh | Ml] (128 pixels x 2K) and B = [Wh; Wl] (2K x 2n, K = 2n rounded up
+// to whole MMAs): each product picks its chunks of A and B, so that neither is stored twice. K index
+// 2z + (0: Re, 1: Im) of column z and output 2j + (0: Re, 1: Im) of L_j: a thread's pixel fills 16-byte
+// core-matrix rows from whole complex values, and reads whole complex values of L back. As many
+// CTAs share an SM as its shared memory holds (three for bf16 at 32 columns). Bound by the latency of a
+// tile's loads and stores (28 MB in 17 us at 192 x 192 x 32; 30 us with 2-byte stores, A stored with a
+// second copy of Mh, 4-byte stores of L and one CTA an SM).
 template <class Op>
-__global__ void __launch_bounds__(kTcThreads, 1) k_reproj_tc(const ReprojTcArgs a) {
+__global__ void __launch_bounds__(kTcThreads) k_reproj_tc(const ReprojTcArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int CE = 16 / Op::kBytes;
   constexpr int KI = 2 * CE;
+  constexpr int CZ = CE / 2;               // columns of a core-matrix row
   const int n = a.g.nc;
   const int N = round_up(2 * n, 16);
-  const int K = round_up(6 * n, KI);
-  const int KC = K / CE;
+  const int K = round_up(2 * n, KI);
+  const int KC = 2 * K / CE;               // chunks: hi, then lo
   const uint32_t BB = (uint32_t)(N / 8) * KC * 128u;   // B bytes
   const uint32_t AB = 16u * KC * 128u;                 // A bytes
   unsigned char* Bs = smem;
@@ -299,25 +342,37 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_reproj_tc(const ReprojTcArgs 
     mbar_init(&bar[0], 1);
     fence_mbar_init();
   }
-  for (uint32_t i = tid * 16; i < BB + AB; i += kTcThreads * 16)
-    *reinterpret_cast<uint4*>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
   pdl_trigger();
   pdl_wait();   // W, X and S come from the preceding kernels
   const int conv = a.ctrl ? a.ctrl->converged : 0;
-  __syncthreads();
-  // B^T rows j (output column), K index seg * 2n + k: Wr[k][j] split into hi / lo
-  for (int e = tid; e < 4 * n * n; e += kTcThreads) {
-    const int k = e / (2 * n), j = e - (e / (2 * n)) * (2 * n);
-    const int kk = k < n ? k : k - n, jj = j < n ? j : j - n;
-    const float2 w = a.W[kk * n + jj];
-    const float wr = (k < n) == (j < n) ? w.x : (k < n ? w.y : -w.y);
-    typename Op::T hi, lo;
-    Op::split(wr, hi, lo);
-    st_op<Op>(Bs, core_off<Op>(j, k, KC), hi);
-    st_op<Op>(Bs, core_off<Op>(j, 2 * n + k, KC), lo);
-    st_op<Op>(Bs, core_off<Op>(j, 4 * n + k, KC), hi);
+  // the first tile's loads are on their way while B is built
+  float2 m[kMaxNc];
+  auto load_tile = [&](int tile) {
+    const long long r = (long long)tile * kTcTile + tid;
+#pragma unroll
+    for (int z = 0; z < kMaxNc; ++z) m[z] = z < n && r < nr ? a.X[z * nr + r] : make_float2(0.f, 0.f);
+    if (a.S) {
+#pragma unroll
+      for (int z = 0; z < kMaxNc; ++z)
+        if (z < n && r < nr) m[z] = csub(m[z], a.S[z * nr + r]);
+    }
+  };
+  if (!conv && blockIdx.x < ntiles) load_tile(blockIdx.x);
+  // B^T rows 2j + cj (output), K index 2z + cz: Re L = Re M Re W - Im M Im W, Im L = Re M Im W + Im M Re W;
+  // zero past the 2n rows and columns
+#pragma unroll 4
+  for (int e = tid; e < N * K / 2; e += kTcThreads) {
+    const int j2 = e / (K / 2), z = e - j2 * (K / 2);
+    const float2 w = z < n && j2 < 2 * n ? a.W[z * n + (j2 >> 1)] : make_float2(0.f, 0.f);
+    const float v0 = (j2 & 1) ? w.y : w.x, v1 = (j2 & 1) ? w.x : -w.y;   // of Re M, of Im M
+    typename Op::T h0, l0, h1, l1;
+    Op::split(v0, h0, l0);
+    Op::split(v1, h1, l1);
+    st_op<Op>(Bs, core_off<Op>(j2, 2 * z, KC), h0);
+    st_op<Op>(Bs, core_off<Op>(j2, 2 * z + 1, KC), h1);
+    st_op<Op>(Bs, core_off<Op>(j2, K + 2 * z, KC), l0);
+    st_op<Op>(Bs, core_off<Op>(j2, K + 2 * z + 1, KC), l1);
   }
-  fence_proxy_async();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -329,35 +384,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_reproj_tc(const ReprojTcArgs 
   bool bad = false;
   for (int tile = blockIdx.x; tile < ntiles && !conv; tile += gridDim.x, ++it) {
     const long long r = (long long)tile * kTcTile + tid;
-    float2 m[kMaxNc];
+    if (it > 0) load_tile(tile);
 #pragma unroll
-    for (int z = 0; z < kMaxNc; ++z) {
-      m[z] = make_float2(0.f, 0.f);
-      if (z < n && r < nr) m[z] = a.S ? csub(a.X[z * nr + r], a.S[z * nr + r]) : a.X[z * nr + r];
-    }
+    for (int q = 0; q < kMaxNc / CZ; ++q) {
+      if (q * CE < K) {
+        typename Op::T hi[CE], lo[CE];
 #pragma unroll
-    for (int z = 0; z < kMaxNc; ++z) {
-      if (z < n) {
-        typename Op::T rh, rl, ih, il;
-        Op::split(m[z].x, rh, rl);
-        Op::split(m[z].y, ih, il);
-        st_op<Op>(As, core_off<Op>(tid, z, KC), rh);
-        st_op<Op>(As, core_off<Op>(tid, n + z, KC), ih);
-        st_op<Op>(As, core_off<Op>(tid, 2 * n + z, KC), rh);
-        st_op<Op>(As, core_off<Op>(tid, 3 * n + z, KC), ih);
-        st_op<Op>(As, core_off<Op>(tid, 4 * n + z, KC), rl);
-        st_op<Op>(As, core_off<Op>(tid, 5 * n + z, KC), il);
+        for (int i = 0; i < CZ; ++i) {
+          Op::split(m[q * CZ + i].x, hi[2 * i], lo[2 * i]);
+          Op::split(m[q * CZ + i].y, hi[2 * i + 1], lo[2 * i + 1]);
+        }
+        *reinterpret_cast<uint4*>(As + core_off<Op>(tid, q * CE, KC)) = Op::pack(hi);
+        *reinterpret_cast<uint4*>(As + core_off<Op>(tid, K + q * CE, KC)) = Op::pack(lo);
       }
     }
-    fence_proxy_async();
+    fence_proxy_async();   // (the first tile's covers the stores of B as well)
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t abase = smem_u32(As), bbase = smem_u32(Bs);
+      const uint32_t ab = smem_u32(As), bb = smem_u32(Bs), lo = (uint32_t)(K / KI) * 256u;
+      const uint32_t asel[3] = {0u, 0u, lo}, bsel[3] = {0u, lo, 0u};
 #pragma unroll 1
-      for (int k = 0; k < K / KI; ++k)
-        tc_mma<Op::kFmt>(tmem, smem_desc(abase + k * 256, 128, KC * 128), smem_desc(bbase + k * 256, 128, KC * 128),
-                         idesc, k > 0 ? 1u : 0u);
+      for (int p = 0; p < 3; ++p)
+#pragma unroll 1
+        for (int k = 0; k < K / KI; ++k)
+          tc_mma<Op::kFmt>(tmem, smem_desc(ab + asel[p] + k * 256, 128, KC * 128),
+                           smem_desc(bb + bsel[p] + k * 256, 128, KC * 128), idesc, (p > 0 || k > 0) ? 1u : 0u);
       tc_commit(&bar[0]);
     }
     if (!mbar_wait_bounded(&bar[0], (unsigned)(it & 1), errp)) bad = true;
@@ -366,19 +418,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_reproj_tc(const ReprojTcArgs 
       bad = true;
       break;
     }
-    // D row of this pixel: columns j < n are Re L[j], n <= j < 2n are Im L[j - n]
-    float* Lf = reinterpret_cast<float*>(a.Lnew);
+    // D row of this pixel: columns 2j, 2j + 1 are L_j
     for (int c0 = 0; c0 < N; c0 += 16) {
       float t[16];
       tmem_ld16(lane_addr + c0, t);
       if (r < nr) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int j = c0 + q;
-          if (j < 2 * n) {
-            const int z = j < n ? j : j - n;
-            Lf[2 * (z * nr + r) + (j < n ? 0 : 1)] = t[q];
-          }
+        for (int q = 0; q < 8; ++q) {
+          const int j = c0 / 2 + q;
+          if (j < n) a.Lnew[j * nr + r] = make_float2(t[2 * q], t[2 * q + 1]);
         }
       }
     }
@@ -399,7 +447,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_reproj_tc(const ReprojTcArgs 
 int gram_tc_parts(const Geom& g) {
   const long long nr = (long long)g.nx * g.ny;
   const int ntiles = (int)((nr + kTcTile - 1) / kTcTile);
-  return ntiles < 148 ? ntiles : 148;
+  const int most = g.nx > 148 ? g.nx : 148;
+  return ntiles < most ? ntiles : most;
 }
 
 size_t gram_tc_smem(int precision) {
@@ -413,8 +462,8 @@ size_t reproj_tc_smem(const Geom& g, int precision) {
   const int ce = 16 / bytes, ki = 2 * ce;
   const int n = g.nc;
   const int N = (2 * n + 15) / 16 * 16;
-  const int K = (6 * n + ki - 1) / ki * ki;
-  const int kc = K / ce;
+  const int K = (2 * n + ki - 1) / ki * ki;
+  const int kc = 2 * K / ce;
   return (size_t)(N / 8) * kc * 128 + 16u * kc * 128 + 64;
 }
 
@@ -427,7 +476,7 @@ static cudaError_t launch_gram_op(const GramTcArgs& a, int precision, cudaStream
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  cudaError_t e = launch_pdl(k_gram_tc<Op>, dim3(gram_tc_parts(a.g)), dim3(kTcThreads), smem, st, a);
+  cudaError_t e = launch_pdl(k_gram_tc<Op>, dim3(gram_tc_parts(a.g)), dim3(kGramTcThreads), smem, st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -449,7 +498,7 @@ static cudaError_t launch_reproj_op(const ReprojTcArgs& a, int precision, cudaSt
   }
   const long long nr = (long long)a.g.nx * a.g.ny;
   const int ntiles = (int)((nr + kTcTile - 1) / kTcTile);
-  const int grid = ntiles < 148 ? ntiles : 148;
+  const int grid = ntiles < 3 * 152 ? ntiles : 3 * 152;   // about what shares the SMs; more go on from tile to tile
   cudaError_t e = launch_pdl(k_reproj_tc<Op>, dim3(grid), dim3(kTcThreads), smem, st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

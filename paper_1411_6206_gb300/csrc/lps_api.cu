@@ -12,8 +12,6 @@
 using namespace lps;
 
 namespace lps {
-cudaError_t launch_gram_plane(const float2* X, const float2* S, const Geom& g, float2* gram_part, int nparts,
-                              cudaStream_t st);
 cudaError_t launch_combine(const float2* L, const float2* S, float2* out, long long n, cudaStream_t st);
 }  // namespace lps
 
@@ -1204,7 +1202,7 @@ int lps_set_state(lps_plan* P, const void* X, const void* S, const void* L_prev,
   if (P->p.precision != LPS_FP32)
     LK(launch_gram_tc(gram_tc_args(P, P->S, false), P->p.precision, P->st));
   else
-    LK(launch_gram_plane(P->X, P->S, P->g, P->gram_part, dc_gram_parts(P->g), P->st));
+    LK(launch_gram_f32(P->X, P->S, P->g, P->gram_part, dc_gram_parts(P->g), P->st));
   CK(cudaStreamSynchronize(P->st));
   P->state_ready = true;
   P->iters_done = iters_done;
@@ -1224,8 +1222,8 @@ int lps_casorati_gram(lps_plan* P, const void* X, const void* S, void* G) {
     LK(launch_gram_tc(a, P->p.precision, P->st));
     nparts = gram_tc_parts(P->g);
   } else {
-    nparts = P->g.nx;
-    LK(launch_gram_plane((const float2*)X, (const float2*)S, P->g, P->gram_part, nparts, P->st));
+    nparts = std::min(P->g.nx, 152);   // a CTA an SM
+    LK(launch_gram_f32((const float2*)X, (const float2*)S, P->g, P->gram_part, nparts, P->st));
   }
   LK(launch_gram_sum(P->gram_part, nparts, P->g.nc, (float2*)G, P->st));
   return LPS_OK;

@@ -241,6 +241,8 @@ cudaError_t launch_dc_persist(const DcArgs* table, const int* start, int nm, int
 cudaError_t launch_dc_reg(const DcArgs& a, cudaStream_t st);
 int dc_gram_parts(const Geom& g);
 int gram_tc_parts(const Geom& g);
+cudaError_t launch_gram_f32(const float2* X, const float2* S, const Geom& g, float2* gram_part, int nparts,
+                            cudaStream_t st);
 cudaError_t launch_gram_sum(const float2* part, int nparts, int nc, float2* G, cudaStream_t st);
 // Rounds n complex values to half precision: h = the rounded pairs, c rewritten with their
 // float32 values (so that every kernel reads the same maps).
@@ -292,6 +294,15 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
 }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+// t + s a as one packed instruction (each half rounds as fmaf does)
+__device__ __forceinline__ float2 fma2(float2 a, float s, float2 t) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z, w;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %4};\n mov.b64 z, {%5, %6};\n"
+      " fma.rn.f32x2 w, x, y, z;\n mov.b64 {%0, %1}, w;\n}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(s), "f"(t.x), "f"(t.y));
+  return r;
+}
 __device__ __forceinline__ float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 // multiply by -i (forward) or +i (inverse)
