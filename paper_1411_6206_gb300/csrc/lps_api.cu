@@ -191,6 +191,9 @@ int gram_parts(const Geom& g, int precision) {
 }
 int gram_part_capacity(const Geom& g) { return std::max(g.nx, gram_tc_parts(g)); }
 
+// Offset in the pinned control copy of the statistics that lps_data_consistency's kernel writes there.
+constexpr size_t kHostPart = (sizeof(DevCtrl) + 255) / 256 * 256;
+
 // Row tasks (where the plane has them), line positions and raster numbers of a mask.
 size_t line_table_bytes(const Geom& g) {
   const size_t lines = (size_t)g.plane * sizeof(int);
@@ -871,7 +874,7 @@ int lps_plan_create(const lps_params* p, void* stream, lps_plan** out) {
   if ((rc = aalloc(P, &P->sup_out, support_words(g)))) return fail(rc);
   if ((rc = aalloc(P, &P->sup_out2, support_words(g)))) return fail(rc);
   if ((rc = aalloc(P, &P->sup_prior, support_words(g)))) return fail(rc);
-  if (cudaMallocHost((void**)&P->h_ctrl, sizeof(DevCtrl)) != cudaSuccess ||
+  if (cudaMallocHost((void**)&P->h_ctrl, kHostPart + (size_t)g.nx * 4 * sizeof(float)) != cudaSuccess ||
       cudaMallocHost((void**)&P->h_persist_slots, lps_plan::kSlots * sizeof(DevPersist)) != cudaSuccess ||
       cudaMallocHost((void**)&P->h_lines_slots, (size_t)lps_plan::kSlots * line_table_bytes(g)) != cudaSuccess) {
     set_err("pinned host allocation failed");
@@ -1331,7 +1334,10 @@ int lps_data_consistency(lps_plan* P, const void* Z, void* X, double* resid_norm
   a.L = src;
   a.S = nullptr;
   a.X = dst;
-  a.dc_part = P->dc_part;
+  // the planes' residuals go straight to pinned host memory (16 bytes a plane, written over the link
+  // while the kernel runs) instead of through a copy: the call is a launch and a wait
+  float* part = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(P->h_ctrl) + kHostPart);
+  a.dc_part = resid_norm2 ? part : P->dc_part;
   const int stall = P->stall_polls;
   P->stall_polls = 0;
   if (stall) {
@@ -1353,8 +1359,6 @@ int lps_data_consistency(lps_plan* P, const void* Z, void* X, double* resid_norm
   }
   if (!dev) CK(cudaMemcpyAsync(X, P->R, img, cudaMemcpyDefault, P->st));
   if (resid_norm2) {
-    std::vector<float> part((size_t)P->g.nx * 4);
-    CK(cudaMemcpyAsync(part.data(), P->dc_part, part.size() * sizeof(float), cudaMemcpyDeviceToHost, P->st));
     CK(cudaStreamSynchronize(P->st));
     double s = 0;
     for (int i = 0; i < P->g.nx; ++i) s += part[(size_t)i * 4];
