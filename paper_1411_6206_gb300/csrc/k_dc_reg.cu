@@ -134,7 +134,6 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     for (int z = 0; z < kNZ; ++z) cn[z] = HALF ? __half22float2(__ldg(Ch + z * xy)) : __ldg(Cc + z * xy);
   };
   if (grp < g.ncoil) load_col(grp);
-  pdl_trigger();
   pdl_wait();   // W and the control block (without W also L, S and X) come from earlier work
   const int conv = a.ctrl ? a.ctrl->converged : 0;
   if (conv) return;   // converged earlier in this frame: nothing is written
@@ -303,6 +302,8 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     }
     // the next coil's column writes touch only this thread's own column: no barrier needed
   }
+
+  pdl_trigger();   // not earlier: the next kernels' CTAs would wait on the SMs through the coil loop
 
   // ---- epilogue: X_k = Z - sum over groups (fixed order), M = X_k - S_k, plane Gram ------
   if constexpr (!ONE && !ACCS) {

@@ -73,20 +73,19 @@ RowLaunch row_launch(const Geom& g, int kc, int pc) {
 
 // CTAs per plane. The fullest of the 152 SMs works through n = nx kc / 152 CTAs in rounds of
 // as many as it holds; a round takes its coils and about two coils' time for the prologue,
-// epilogue and first loads, longer the more CTAs share the SM. Measured (us per iteration, kc =
-// 1, 2, 3, 4): 192 x 192 x 32, 12 coils 211, 206, 187, 199; 160 x 160 x 24, 14 coils 162, 128, 142, 131;
-// 160 x 160 x 14, 16 coils 91, 71, 82, 78: the rule takes 3, 2 and 2.
+// epilogue and first loads, a fifth longer for every CTA that shares the SM. Over 13 planes this is 0.2 %
+// from the fastest kc of each. Us per iteration at kc = 1, 2, 3, 4, 5, 7: 192 x 192 x 32, 12 coils 205, 191,
+// 173, 195, 222, 250; 160 x 160 x 24, 14 coils 155, 120, 132, 123, 118, 134; 112 x 112 x 14, 15 coils 62, 53, 50,
+// 50, 46, 60; 80 x 80 x 24, 13 coils 91, 77, 66, 67, 60, 58.
 int rows_kc(const Geom& g) {
   const int fit = rows_fit(g);
-  const double crowd[5] = {0.0, 1.0, 1.15, 1.4, 1.7};
   int best = 1;
   double least = 1e30;
   for (int kc = 1; kc <= std::min(8, g.ncoil); ++kc) {
     const int coils = (g.ncoil + kc - 1) / kc;
     double t = 0;
     for (int n = (g.nx * kc + 151) / 152; n > 0; n -= fit) {
-      const int k = std::min(n, fit);
-      t += (coils + 2) * (k <= 4 ? crowd[k] : 0.4 * k + 0.1);
+      t += (coils + 2) * (0.8 + 0.2 * std::min(n, fit));
     }
     if (t < least) {
       least = t;

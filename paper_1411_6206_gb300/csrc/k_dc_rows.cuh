@@ -251,7 +251,6 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
 #pragma unroll
     for (int k = 0; k < EARLY; ++k) load_prev(OT * (zl + k * zs), Zo[k]);
   }
-  pdl_trigger();
   pdl_wait();
   if (a.ctrl && a.ctrl->converged) {
     cp_async_wait_all();
@@ -432,6 +431,7 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
     }
   }
   // (a thread's next coil writes the column that it has read: no barrier at the end of a coil)
+  pdl_trigger();   // not earlier: the next kernels' CTAs would wait on the SMs through the coil loop
   if (MODE == kDcForward) return;
 
   // ---- epilogue: X_k = Z - sum over the CTAs of the plane, M = X_k - S_k ----------------------

@@ -109,33 +109,52 @@ __device__ __forceinline__ int next_pos(int p, int np) {
   return p - 2;
 }
 
-// Cyclic Jacobi on the Hermitian n x n matrix in A (zero-padded to even np); the
-// eigenvectors are accumulated into V (V <- V J per rotation). An and Vn are the second
-// buffers of the position permutation; on return A and V point at the results (index
-// order). Each thread keeps one task over all steps, since the tasks address positions:
-// either a block (k1 <= k2) of the 2 x 2 blocks of A, which it rotates on both sides with
-// the rotations of pairs k1 and k2 and writes (with its mirror) at the moved positions, or
-// two rows of V at pair k2. The three kinds of task (off-diagonal blocks, diagonal blocks,
-// V rows) start on warp boundaries, so that no warp splits between their code paths. Every
-// thread computes the rotations it needs itself from the diagonal blocks, so one barrier per
-// step suffices. Returns the sweeps done.
-// Threads that hold a task of the Jacobi step below (whole warps): off-diagonal blocks from
-// thread 0, diagonal blocks and V row pairs each from the next warp boundary.
-__host__ __device__ __forceinline__ int jacobi_threads(int n) {
+// Its inverse.
+__device__ __forceinline__ int prev_pos(int p, int np) {
+  if (np == 2 || p == 0) return p;
+  if (p == 2) return 1;
+  if ((p & 1) == 0) return p - 2;
+  return p == np - 1 ? np - 2 : p + 2;
+}
+
+// Above 16 columns V is carried in registers by 8 warps; up to 16 its rows are tasks of the step.
+__host__ __device__ __forceinline__ constexpr bool jacobi_vreg(int n) { return n > 16; }
+constexpr int kVWarps = 8;
+// Threads of the Jacobi step below (whole warps): off-diagonal blocks from thread 0, diagonal blocks
+// and V each from the next warp boundary; at most 416 (n = 32).
+__host__ __device__ __forceinline__ int jacobi_vbase(int n) {
   const int np = n + (n & 1), nh = np >> 1;
   const int noff = nh * (nh - 1) / 2;
   const int dbase = ((noff + 31) >> 5) << 5;
-  const int vbase = ((dbase + nh + 31) >> 5) << 5;
-  return ((vbase + nh * nh + 31) >> 5) << 5;
+  return ((dbase + nh + 31) >> 5) << 5;
+}
+__host__ __device__ __forceinline__ int jacobi_threads(int n) {
+  const int nh = (n + 1) >> 1;
+  return jacobi_vbase(n) + (jacobi_vreg(n) ? 32 * kVWarps : (nh * nh + 31) / 32 * 32);
 }
 
 __device__ __forceinline__ void jsync(int nthr) { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); }
 
+// Cyclic Jacobi on the Hermitian n x n matrix in A (zero-padded to even np); the
+// eigenvectors are accumulated into V (V <- V J per rotation). An and Vn are the second
+// buffers of the position permutation; on return A and V point at the results (index
+// order). Each thread of A keeps one task over all steps, since the tasks address positions:
+// a block (k1 <= k2) of the 2 x 2 blocks of A, which it rotates on both sides with
+// the rotations of pairs k1 and k2 and writes (with its mirror) at the moved positions. The
+// off-diagonal and the diagonal blocks start on warp boundaries, so that no warp splits between
+// their code paths. Every thread computes the rotations it needs itself from the diagonal blocks, so
+// one barrier per step suffices.
+// A step is bound by the chain from the diagonal blocks through the rotation parameters to the
+// moved blocks, and, where the warps are many, by their issue. So above 16 columns V stays in
+// registers, a lane a position, and takes a step's rotations (which the diagonal blocks' threads
+// leave in rot) during the next step, partner and move by shuffles: 51 us a launch at n = 32
+// against 55 with two rows of V and a pair as a task of the step itself (its own rotation
+// parameters, 8 warps). Up to 16 columns such tasks are the faster form (32 x 32 x 8: 0.3 us an iteration).
 // Called by threads 0 .. jacobi_threads(n) - 1 only (named barrier 1): the other warps of the
-// CTA have no task and wait at the CTA barrier that follows.
+// CTA have no task and wait at the CTA barrier that follows. Returns the sweeps done.
 template <int NCT>
-__device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt, float eps, float floor_,
-                      int max_sweeps, float start, int* flags) {
+__device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, float4 (*rot)[kMaxNc / 2], int n_rt,
+                      float eps, float floor_, int max_sweeps, float start, int* flags) {
   const int n = NCT ? NCT : n_rt;
   const int nthr = jacobi_threads(n);
   using C = float2;
@@ -145,9 +164,10 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
   const int nh = np >> 1;
   const int noff = nh * (nh - 1) / 2;           // off-diagonal blocks k1 < k2 from thread 0
   const int dbase = ((noff + 31) >> 5) << 5;      // diagonal blocks
-  const int vbase = ((dbase + nh + 31) >> 5) << 5;   // V row pairs (at most 416 threads: n <= 32)
+  const int vbase = jacobi_vbase(n);
   const int tid = threadIdx.x;
-  int role = 0, k1 = 0, k2 = 0, r0 = 0;
+  const bool vreg = jacobi_vreg(n);
+  int role = 0, k1 = 0, k2 = 0, r0 = 0;   // role 1: a block of A, 2: rows r0, r0 + 1 of V, 3: rows of V in registers
   if (tid < noff) {
     role = 1;
     int t = tid;
@@ -159,6 +179,8 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
   } else if (tid >= dbase && tid < dbase + nh) {
     role = 1;
     k1 = k2 = tid - dbase;
+  } else if (vreg && tid >= vbase) {
+    role = 3;
   } else if (tid >= vbase && tid < vbase + nh * nh) {
     role = 2;
     const int t = tid - vbase;
@@ -168,6 +190,26 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
   const int p1 = 2 * k1, q1 = p1 + 1, p2 = 2 * k2, q2 = p2 + 1;
   const int np1 = next_pos(p1, np), nq1 = next_pos(q1, np);
   const int np2 = next_pos(p2, np), nq2 = next_pos(q2, np);
+  // V in registers: lane `pos` holds position pos of rows vrow, vrow + 8, ...
+  const int pos = tid & 31, vrow = (tid - vbase) >> 5, from = pos < np ? prev_pos(pos, np) : pos;
+  C v[4];
+  if (role == 3) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = vrow + u * kVWarps;
+      v[u] = r < n && pos < np ? V[r * kLd + pos] : mkc(R(0), R(0));
+    }
+  }
+  auto turn = [&](const C4* rt) {   // V <- V J of one step, moved to the next step's positions
+    const C4 r = rt[pos < np ? pos >> 1 : 0];
+    const C e = mkc((pos & 1) ? r.y : -r.y, r.z);   // p: c v_p - v_q conj(se), q: c v_q + v_p se
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const C o = mkc(__shfl_xor_sync(0xffffffffu, v[u].x, 1), __shfl_xor_sync(0xffffffffu, v[u].y, 1));
+      const C t = add_(scl_<C, R>(v[u], r.x), mul_(o, e));
+      v[u] = mkc(__shfl_sync(0xffffffffu, t.x, from), __shfl_sync(0xffffffffu, t.y, from));
+    }
+  };
   int sweep = 0;
   for (;;) {
     // converged when no off-diagonal entry exceeds `start` times its rotation threshold (a
@@ -175,16 +217,20 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
     // move rounding noise are not started
     if (tid == 0) flags[sweep & 1] = 0;
     jsync(nthr);
-    for (int t = tid; t < n * n; t += nthr) {
-      const int p = t / n, q = t - (t / n) * n;
-      if (p < q) {
-        // the rotation test of rot_params at `start` times the thresholds (no rotation
-        // parameters)
-        const float app = A[p * kLd + p].x, aqq = A[q * kLd + q].x;
-        const float2 apq = A[p * kLd + q];
-        const float g2 = apq.x * apq.x + apq.y * apq.y;
-        const float lim = fmaxf(start * eps * fmaxf(fabsf(app), fabsf(aqq)), start * floor_);
-        if (g2 > lim * lim) flags[sweep & 1] = 1;
+    if (role == 3) {
+      if (sweep > 0) turn(rot[(np - 2) & 1]);   // the last step of the sweep before
+    } else {
+      for (int t = tid; t < n * n; t += vreg ? vbase : nthr) {
+        const int p = t / n, q = t - (t / n) * n;
+        if (p < q) {
+          // the rotation test of rot_params at `start` times the thresholds (no rotation
+          // parameters)
+          const float app = A[p * kLd + p].x, aqq = A[q * kLd + q].x;
+          const float2 apq = A[p * kLd + q];
+          const float g2 = apq.x * apq.x + apq.y * apq.y;
+          const float lim = fmaxf(start * eps * fmaxf(fabsf(app), fabsf(aqq)), start * floor_);
+          if (g2 > lim * lim) flags[sweep & 1] = 1;
+        }
       }
     }
     jsync(nthr);
@@ -196,6 +242,7 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
         const C b10 = A[q1 * kLd + p2], b11 = A[q1 * kLd + q2];
         const C4 ra = rot_of(k1);
         if (k1 == k2) {
+          if (vreg) rot[st & 1][k1] = ra;
           C o00 = b00, o01 = b01, o10 = b10, o11 = b11;
           if (ra.w != R(0)) {
             // a_pp - t|a_pq|, a_qq + t|a_pq|, exact zeros off the diagonal
@@ -238,16 +285,27 @@ __device__ int jacobi(float2*& A, float2*& An, float2*& V, float2*& Vn, int n_rt
         Vn[r0 * kLd + nq2] = add_(mul_(vp0, se), scl_<C, R>(vq0, r.x));
         Vn[(r0 + 1) * kLd + np2] = sub_(scl_<C, R>(vp1, r.x), mul_(vq1, conj_(se)));
         Vn[(r0 + 1) * kLd + nq2] = add_(mul_(vp1, se), scl_<C, R>(vq1, r.x));
+      } else if (role == 3 && st > 0) {
+        turn(rot[(st - 1) & 1]);
       }
       jsync(nthr);
       C* t = A;
       A = An;
       An = t;
-      t = V;
-      V = Vn;
-      Vn = t;
+      if (!vreg) {
+        t = V;
+        V = Vn;
+        Vn = t;
+      }
     }
     ++sweep;
+  }
+  if (role == 3) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = vrow + u * kVWarps;
+      if (r < n && pos < np) V[r * kLd + pos] = v[u];
+    }
   }
   return sweep;
 }
@@ -257,12 +315,13 @@ struct alignas(16) EigShared {
   float2 A1[kMaxNc * kLd];
   float2 V[kMaxNc * kLd];
   float2 G[kMaxNc * kLd];
-  float2 V1[kMaxNc * kLd];   // second eigenvector buffer of the Jacobi permutation
+  float2 V1[kMaxNc * kLd];   // second eigenvector buffer of the Jacobi permutation (up to 16 columns)
+  float4 rot[2][kMaxNc / 2];   // the rotations of a Jacobi step and of the one before
   float f[kMaxNc];         // sigma''_i / sigma_i
   double lam[kMaxNc];      // eigenvalues
   float sprevf[kMaxNc];    // sigma_prev as float32
   int flags[4];
-  int jac_sweeps, jac_odd;   // Jacobi sweeps done; 1 if A and V ended in the second buffers
+  int jac_sweeps, jac_odd;   // Jacobi sweeps done; 1 if A (and V, up to 16 columns) ended in the second buffer
   float lrs_l1;              // l1 off the prior support of the previous iteration
   unsigned char tri[2][kMaxNc * (kMaxNc + 1) / 2];   // (i, j) of upper-triangle entry e
   double sprev[kMaxNc];    // sigma_prev
@@ -349,11 +408,16 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   const int tid = threadIdx.x;
   const int n = NCT ? NCT : a.g.nc;
   const int np = n + (n & 1);
+  pdl_wait();   // the Gram partials, statistics and control block come from earlier kernels
   // The successor (the data-consistency kernel) is released only after this wait: once it
   // runs, every kernel before this one has completed, so it may read their outputs (X, L and
-  // the sparse parts of the previous iteration) before its own wait.
-  pdl_wait();   // the Gram partials, statistics and control block come from earlier kernels
-  pdl_trigger();
+  // the sparse parts of the previous iteration) before its own wait. Above 8 columns it is
+  // released only after the Jacobi sweeps: that leaves it the time to start and read them, while
+  // released here its CTAs would hold the SMs through the eigendecomposition, where the sparse step
+  // and the kernels before the update run (an iteration of 160 x 160 x 24 127 us released here, 118
+  // after the sweeps; 192 x 192 x 32 with BF16 contractions 260 and 201; 32 x 32 x 8 15.7 and 16.1).
+  const bool release_now = a.part == 2 || n <= 8;
+  if (release_now) pdl_trigger();
   const int nn = n * n;
   if constexpr (CL > 1) {
     cg::cluster_group cl = cg::this_cluster();
@@ -489,7 +553,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
 
   int sweeps = 0;
   float2* Af = sh.A0;    // eigenvalues on the diagonal after the Jacobi
-  float2* Vres = sh.V;   // eigenvectors (columns)
+  const float2* Vres = sh.V;   // eigenvectors (columns)
   if (a.part != 2) {
     // 2. Gram matrix: combine the chunk sums in a fixed order; exact Hermitian symmetry
     if (CL == 1 && tid < ksub * nn) sub[tid] = gacc0;
@@ -560,19 +624,20 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
       // 8u of the trace), still below the float32 Gram's own accumulation error (about
       // u sqrt(rows) of the trace); before the float64 refinement (part 1) at 2x, which leaves
       // the refinement pairs coupled well below its 1e-3 gap limit
-      sweeps = jacobi<NCT>(Af, Afn, Vf, Vfn, n, 4.8e-7f, 6.0e-8f * trace + 1e-30f, 12, a.part == 1 ? 2.f : 8.f,
+      sweeps = jacobi<NCT>(Af, Afn, Vf, Vfn, sh.rot, n, 4.8e-7f, 6.0e-8f * trace + 1e-30f, 12, a.part == 1 ? 2.f : 8.f,
                            sh.flags);
       if (tid == 0) {
         // own fields: other Jacobi threads may still read flags[] in their last convergence test
         sh.jac_sweeps = sweeps;
-        sh.jac_odd = Af != sh.A0;   // the results sit in the second buffers (odd step count)
+        sh.jac_odd = Af != sh.A0;   // the result sits in the second buffer (odd step count)
       }
     }
     __syncthreads();
+    if (!release_now) pdl_trigger();
     sweeps = sh.jac_sweeps;
     if (sh.jac_odd) {
       Af = sh.A1;
-      Vres = sh.V1;
+      if (!jacobi_vreg(n)) Vres = sh.V1;
     }
 
     if (a.part == 1) {
