@@ -458,12 +458,10 @@ GramTcArgs gram_tc_args(lps_plan* P, const float2* S, bool with_ctrl = true) {
 
 // Step (0): X_0 = E^H d, L_0 := X_0, S_0 = 0, Gram of X_0, max |T(X_0)|.
 int enqueue_init(lps_plan* P, cudaStream_t st) {
-  CK(cudaMemsetAsync(P->ctrl, 0, sizeof(DevCtrl), st));
-  // an inactive batch member starts "converged": every kernel of the frame returns at once
-  CK(cudaMemcpyAsync(&P->ctrl->converged, &P->persist->skip, sizeof(int), cudaMemcpyDeviceToDevice, st));
-  // Each frame starts its eigendecomposition from scratch unless the plan reconstructs a
-  // sequence, where the previous frame's eigenvectors are the warm start.
-  if (!P->p.recursive) CK(cudaMemsetAsync(&P->persist->v_valid, 0, sizeof(int), st));
+  // The control block, cleared; an inactive batch member starts "converged": every kernel of the
+  // frame returns at once. Each frame starts its eigendecomposition from scratch unless the plan
+  // reconstructs a sequence, where the previous frame's eigenvectors are the warm start.
+  LK(launch_frame_begin(P->ctrl, P->persist, P->p.recursive != 0, st));
   const bool tc = P->p.precision != LPS_FP32;
   DcArgs a = dc_args(P);
   a.X = P->X;

@@ -247,6 +247,7 @@ cudaError_t launch_gram_sum(const float2* part, int nparts, int nc, float2* G, c
 // Rounds n complex values to half precision: h = the rounded pairs, c rewritten with their
 // float32 values (so that every kernel reads the same maps).
 cudaError_t launch_round_half(float2* c, __half2* h, long long n, cudaStream_t st);
+cudaError_t launch_frame_begin(DevCtrl* ctrl, DevPersist* persist, bool keep_v, cudaStream_t st);
 cudaError_t launch_settle(const DevCtrl* ctrl, int k0, float2* S0, const float2* S1, long long n, uint32_t* sup0,
                           const uint32_t* sup1, long long nw, float* part0, const float* part1, int np,
                           cudaStream_t st);
