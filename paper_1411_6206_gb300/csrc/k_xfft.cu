@@ -6,11 +6,16 @@
 //   forward: hybrid [x][coil][line]   -> k-space [coil][line][kx] (d = F_x h)
 // One CTA transforms kLines lines of one coil; the transpose goes through shared memory
 // so that both the row reads and the x-major writes are contiguous.
-#include "lps_internal.cuh"
+#include "xfft_rows.cuh"
 
 namespace lps {
 
-constexpr int kLines = 16;
+template <> cudaError_t launch_xfft_rows<0>(const XfftArgs&, cudaStream_t);
+template <> cudaError_t launch_xfft_rows<1>(const XfftArgs&, cudaStream_t);
+template <> cudaError_t launch_xfft_rows<2>(const XfftArgs&, cudaStream_t);
+template <> cudaError_t launch_xfft_rows<3>(const XfftArgs&, cudaStream_t);
+
+constexpr int kLines = kXfftLines;
 
 // A plan that holds a slab of the volume (planes x0 .. x0+nx-1 of nxt) transforms whole
 // readouts of nxt samples; the inverse keeps its own planes, the forward takes the planes it
@@ -69,7 +74,13 @@ size_t xfft_smem_bytes(const Geom& g) {
 }
 
 // Grid: (ceil(nlines_cap / kLines), ncoil); CTAs past the current line count exit.
+// Readouts whose length is in the table of dc_rows.cuh take the register transforms (xfft_rows.cuh).
 cudaError_t launch_xfft(const XfftArgs& a, cudaStream_t st) {
+  cudaError_t er = launch_xfft_rows<0>(a, st);
+  if (er == cudaErrorNotSupported) er = launch_xfft_rows<1>(a, st);
+  if (er == cudaErrorNotSupported) er = launch_xfft_rows<2>(a, st);
+  if (er == cudaErrorNotSupported) er = launch_xfft_rows<3>(a, st);
+  if (er != cudaErrorNotSupported) return er;
   const size_t smem = xfft_smem_bytes(a.g);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_xfft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

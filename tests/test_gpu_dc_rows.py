@@ -99,6 +99,42 @@ def test_half_maps_and_samples_read_the_rounded_values(L, nz, nx, ny, nc, fmt):
         assert rel(out[1], ref) < 2e-5        # a sample within rounding of a binary16 tie may go the other way
 
 
+def radix_plan(n):
+    out = []
+    for r in (16, 8, 4, 2, 3, 5, 7):
+        while n % r == 0:
+            out.append(r)
+            n //= r
+    return tuple(out)
+
+
+@pytest.mark.parametrize("half", ["", "coil_format", "data_format"])
+@pytest.mark.parametrize("nz,nx,ny,nc,fz", [(2, 8, 16, 2, 1), (5, 16, 40, 7, 0), (9, 8, 72, 1, 1), (15, 24, 120, 6, 1),
+                                            (14, 16, 160, 5, 0), (20, 8, 96, 4, 1), (21, 8, 168, 3, 1), (24, 8, 240, 2, 1),
+                                            (32, 16, 192, 4, 1)])
+def test_equals_the_runtime_sized_kernel(L, nz, nx, ny, nc, fz, half):
+    """Step (4), E and E^H of the default path against the runtime-sized kernel on the same plan (so on
+    the same rounded maps or samples): two float32 evaluations of one sum, within the operators' bound."""
+    case = make_case(nz, nx, ny, nc, seed=ny + nz, fft_z=fz, frac=0.4)
+    pl = plan_for(L, case, nz, nx, ny, nc, fft_z=fz, **({half: 1} if half else {}))
+    rng = np.random.default_rng(6)
+    Z = dev(c64(rng.standard_normal((nz, nx, ny)) + 1j * rng.standard_normal((nz, nx, ny))))
+    outs = []
+    for generic in (False, True):
+        if generic:
+            L.apply_tune(pl.handle, 2, radix_plan(ny), radix_plan(nz), lrs_tiles=1)
+        X, A = torch.empty_like(Z), torch.empty_like(Z)
+        k = torch.empty((nc, case["nlines"], nx), dtype=torch.complex64, device="cuda")
+        r2 = L.data_consistency(pl.handle, Z, X)
+        L.forward(pl.handle, Z, k)
+        L.adjoint(pl.handle, dev(case["d"]), A)
+        outs.append((X.cpu().numpy(), k.cpu().numpy(), A.cpu().numpy(), r2))
+    for got, want in zip(outs[0][:3], outs[1][:3]):
+        assert rel(got, up(want)) < OP_TOL
+    assert abs(outs[0][3] - outs[1][3]) < 1e-5 * outs[1][3]
+    pl.close()
+
+
 @pytest.mark.parametrize("nz,nx,ny,nc", [(5, 64, 48, 3), (7, 72, 40, 6), (10, 64, 80, 4), (15, 64, 104, 5), (32, 16, 192, 2),
                                          (16, 128, 128, 8)])
 def test_first_frame_equals_later_frames(L, nz, nx, ny, nc):
