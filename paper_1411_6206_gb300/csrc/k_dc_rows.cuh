@@ -216,15 +216,19 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
 #pragma unroll
     for (int z = 0; z < nz; ++z) cp_async8(buf + z * rs + pos, C + z * xy);
   };
-  // The maps, the samples and the mask were complete before any kernel that can release this one
-  // started (nothing that writes them lets its successor start early): the first coil's are copied
-  // before the wait, its map column unless the rows hold M first.
+  // In a frame (ctrl) the maps and the samples were complete before its first kernel started: the
+  // first coil's are copied before the wait, its map column unless the rows hold M first. A call of
+  // one operator may directly follow the kernel that wrote them and copies them after it.
   float2* Msh = WS ? acc : buf;
   auto stage_first_map = [&]() {
     if (MODE != kDcAdjoint && col && !half_maps) stage_map(map_col(rank));
   };
-  if (staged) stage_samples(rank);
-  if (WS || !early) stage_first_map();
+  const bool ahead = a.ctrl != nullptr;
+  auto stage_first = [&]() {
+    if (staged) stage_samples(rank);
+    if (WS || !early) stage_first_map();
+  };
+  if (ahead) stage_first();
   // Iteration form with W: this launch is released by the eigen kernel after that kernel's own
   // wait, so the outputs of the data-consistency kernel before it and of what that one waited for
   // (X_{k-1}, S_{k-1}, L_{k-1}) are read while it still runs: M_{k-1} into shared memory, Z_{k-1} of the
@@ -256,6 +260,7 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
     cp_async_wait_all();
     return;
   }
+  if (!ahead) stage_first();
 
   float dz2 = 0.f, z2 = 0.f, resid = 0.f;   // ||Z_k - Z_{k-1}||^2, ||Z_{k-1}||^2, ||E Z - d||^2: this thread's share
   const float2* Z = nullptr;

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(16 * (A > B ? A : B)) k_xfft_rows(const XfftAr
   const Geom& g = a.g;
   const int tid = threadIdx.x, c = blockIdx.y, l0 = blockIdx.x * NL;
   for (int i = tid; i < NX; i += blockDim.x) tw[i] = a.tw_x[i / B * (i % B)];
+  pdl_wait();   // the samples come from the preceding kernel
   const int m = a.persist->nlines;
   if (l0 >= m) return;
   const int nl = min(NL, m - l0), x0 = g.x0, nxl = g.nx;
