@@ -185,9 +185,10 @@ def dc_kernel_name(w, tuned):
         return "k_dc"
     if (w.ny, w.nz) == (128, 16):
         return "k_dc_reg"
-    if (w.ny, w.nz) in ((192, 32), (32, 8)):
+    if (w.ny, w.nz) == (32, 8):
         return "k_dc_fixed"
-    return "k_dc"
+    factors = w.ny % 8 == 0 and (w.ny <= 216 or w.ny in (224, 240, 256))
+    return "k_dc_rows" if factors and w.nz <= 32 else "k_dc"
 
 
 def dc_bytes_per_launch(w, m):
