@@ -223,12 +223,9 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
   auto stage_first_map = [&]() {
     if (MODE != kDcAdjoint && col && !half_maps) stage_map(map_col(rank));
   };
-  const bool ahead = a.ctrl != nullptr;
-  auto stage_first = [&]() {
-    if (staged) stage_samples(rank);
-    if (WS || !early) stage_first_map();
-  };
-  if (ahead) stage_first();
+  if (!a.ctrl) pdl_wait();
+  if (staged) stage_samples(rank);
+  if (WS || !early) stage_first_map();
   // Iteration form with W: this launch is released by the eigen kernel after that kernel's own
   // wait, so the outputs of the data-consistency kernel before it and of what that one waited for
   // (X_{k-1}, S_{k-1}, L_{k-1}) are read while it still runs: M_{k-1} into shared memory, Z_{k-1} of the
@@ -260,7 +257,6 @@ __device__ __forceinline__ void dc_rows_plane(const DcArgs& a, const RowLaunch& 
     cp_async_wait_all();
     return;
   }
-  if (!ahead) stage_first();
 
   float dz2 = 0.f, z2 = 0.f, resid = 0.f;   // ||Z_k - Z_{k-1}||^2, ||Z_{k-1}||^2, ||E Z - d||^2: this thread's share
   const float2* Z = nullptr;
