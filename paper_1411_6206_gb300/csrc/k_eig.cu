@@ -333,6 +333,10 @@ struct alignas(16) EigShared {
 };
 
 
+// The two halves of a meeting of the cluster, by all threads of every CTA (converged warps).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // One chunk sum of a Gram entry over the partials: task = part * nn + e sums partials
 // part, part + ksub, part + 2 ksub, ... of entry e, sixteen loads in flight at a time.
 // Every partial holds an exactly Hermitian matrix and all entries are summed in the same
@@ -364,7 +368,9 @@ __device__ __forceinline__ float2 gram_chunk(const float2* __restrict__ gram_par
 // CTA `rank`'s share of the Gram: ne entries, each summed over the partials in 512 / ne interleaved
 // chunks (a warp reads consecutive entries of a partial), the chunks added in order. Every partial
 // holds an exactly Hermitian matrix and every entry is summed in the same order, so the result is
-// Hermitian too. Ends with the cluster's meeting, after which the first CTA has all of G.
+// Hermitian too. The first CTA's shared memory may be written only once that CTA runs, so the stores
+// stand behind the cluster's first meeting (every CTA arrives at its start). Ends with the second,
+// after which the first CTA has all of G.
 template <int CL>
 __device__ __forceinline__ void gram_share(const EigArgs& a, EigShared& sh, int nn, int n, int rank,
                                            cg::cluster_group cl) {
@@ -388,6 +394,7 @@ __device__ __forceinline__ void gram_share(const EigArgs& a, EigShared& sh, int 
     sub[tid] = s;
   }
   __syncthreads();
+  cluster_wait();
   if (tid < ne && e0 + tid < nn) {
     float2 s = sub[tid];
     for (int q = 1; q < ksub; ++q) s = cadd(s, sub[q * ne + tid]);
@@ -408,6 +415,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
   const int tid = threadIdx.x;
   const int n = NCT ? NCT : a.g.nc;
   const int np = n + (n & 1);
+  if constexpr (CL > 1) cluster_arrive();   // the wait is in gram_share, or before an early return
   pdl_wait();   // the Gram partials, statistics and control block come from earlier kernels
   // The successor (the data-consistency kernel) is released only after this wait: once it
   // runs, every kernel before this one has completed, so it may read their outputs (X, L and
@@ -423,7 +431,10 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     if (rank > 0) {
-      if (ctrl->converged) return;   // set by this launch only after the cluster has met
+      if (ctrl->converged) {   // set by this launch only after the cluster has met a second time
+        cluster_wait();
+        return;
+      }
       gram_share<CL>(a, sh, nn, n, rank, cl);
       return;
     }
@@ -514,7 +525,10 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
     }
   }
   __syncthreads();
-  if (sh.flags[2]) return;
+  if (sh.flags[2]) {
+    if constexpr (CL > 1) cluster_wait();
+    return;
+  }
   if constexpr (CL > 1) gram_share<CL>(a, sh, nn, n, 0, cg::this_cluster());
 
   // 1. statistics record and the stopping rule (the second part of the float64 mode has done it)
