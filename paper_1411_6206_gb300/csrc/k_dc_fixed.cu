@@ -139,7 +139,10 @@ __global__ void __launch_bounds__(NCG* NT, 1) k_dc_fixed(const DcArgs a) {
     for (int z = 0; z < NZ; ++z) bulk_g2s(slot + z * NY, src + z * xy, kRowBytes, b);
   };
   // The first two coil planes of each group are requested before anything else; the
-  // control flag and the other global inputs are loaded while they are in flight.
+  // control flag and the other global inputs are loaded while they are in flight. In a frame (ctrl) the
+  // maps were complete before its first kernel started; a call of one operator may directly follow
+  // the kernel that rounded them and waits for it first.
+  if (!a.ctrl) pdl_wait();
   unsigned inflight = 0;   // slots with a copy in flight (thread gtid == 0 of each group)
   unsigned phase = 0;      // parity of the next phase to wait for, per slot
   if (gtid == 0) {

@@ -123,9 +123,10 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     }
   };
   if (early) prologue_loads();
-  // Coil maps are set before any frame work: the column of this thread for the group's first
-  // coil is loaded now; inside the loop the next coil's column is loaded one coil ahead, so
-  // that its latency passes during the row phase of the current coil.
+  // Coil maps are set before any frame work: in a frame (ctrl) the column of this thread for the
+  // group's first coil is loaded now. A call of one operator may directly follow the kernel that
+  // rounded the maps and loads it after the wait. Inside the loop the next coil's column is loaded
+  // one coil ahead, so that its latency passes during the row phase of the current coil.
   float2 cn[kNZ];
   auto load_col = [&](int c) {
     const float2* Cc = a.coils + (long long)c * g.N + xoff + gt;
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
 #pragma unroll
     for (int z = 0; z < kNZ; ++z) cn[z] = HALF ? __half22float2(__ldg(Ch + z * xy)) : __ldg(Cc + z * xy);
   };
+  if (!a.ctrl) pdl_wait();
   if (grp < g.ncoil) load_col(grp);
   pdl_wait();   // W and the control block (without W also L, S and X) come from earlier work
   const int conv = a.ctrl ? a.ctrl->converged : 0;

@@ -1,5 +1,6 @@
 """Orders in the kernels' sources that no run can show to be missing (a race may never show): another
-CTA's shared memory is touched only behind a meeting of the cluster."""
+CTA's shared memory is touched only behind a meeting of the cluster, and an operator call reads the maps
+and the samples only behind its dependency wait."""
 import os
 import re
 
@@ -44,3 +45,12 @@ def test_eigen_kernel_pairs_its_cluster_barrier():
     for m in re.finditer(r"\breturn;", before):
         near = before[max(0, m.start() - 60):m.start()]
         assert "cluster_wait()" in near or "gram_share<CL>" in near, near
+
+
+@pytest.mark.parametrize("file,function,first_read", [("k_dc_reg.cu", "k_dc_reg", "load_col(grp)"),
+                                                      ("k_dc_fixed.cu", "k_dc_fixed", "issue(grp, "),
+                                                      ("k_dc_rows.cuh", "dc_rows_plane", "stage_samples(rank)")])
+def test_operator_calls_wait_before_they_read_maps_or_samples(file, function, first_read):
+    """Outside a frame (no control block) the call may directly follow the kernel that wrote them."""
+    b = body(code(file), function)
+    assert "if (!a.ctrl) pdl_wait();" in b[:b.index(first_read)]
