@@ -748,6 +748,35 @@ int plan_frame_done(lps_plan* P) {
   frame_done(P);
   return LPS_OK;
 }
+size_t plan_gram_part_bytes(const lps_plan* P) {
+  return (size_t)gram_part_capacity(P->g) * P->g.nc * P->g.nc * sizeof(float2);
+}
+// The launch shapes decide how many Gram partials the data-consistency step leaves for the next eigen
+// kernel, and how many statistic partials the sparse step leaves. A state that is to be iterated
+// further has those of the shapes before: the Gram is formed again (within a run of slabs nothing
+// reads it, their reduced record holds it), the statistics are added up into as many as the new
+// shapes read.
+int plan_set_shapes(lps_plan* P, const Geom& g) {
+  const int gram0 = gram_parts(P->g, P->p.precision), lrs0 = lrs_blocks(P->g);
+  P->g = g;
+  P->graph_valid = false;
+  if (!P->state_ready) return LPS_OK;
+  const int gram1 = gram_parts(P->g, P->p.precision), lrs1 = lrs_blocks(P->g);
+  if (gram1 != gram0) LK(launch_gram_f32(P->X, P->S, P->g, P->gram_part, gram1, P->st));
+  if (lrs1 != lrs0) {
+    std::vector<float> part((size_t)lrs0 * 2), sum((size_t)lrs1 * 2);
+    for (float* p : {P->lrs_part, P->lrs_part2}) {
+      CK(cudaMemcpyAsync(part.data(), p, part.size() * sizeof(float), cudaMemcpyDeviceToHost, P->st));
+      CK(cudaStreamSynchronize(P->st));
+      std::fill(sum.begin(), sum.end(), 0.f);
+      for (int i = 0; i < lrs0; ++i)
+        for (int j = 0; j < 2; ++j) sum[2 * (i % lrs1) + j] += part[2 * i + j];
+      CK(cudaMemcpyAsync(p, sum.data(), sum.size() * sizeof(float), cudaMemcpyHostToDevice, P->st));
+      CK(cudaStreamSynchronize(P->st));
+    }
+  }
+  return LPS_OK;
+}
 DcArgs plan_dc_args(lps_plan* P) { return dc_args(P); }
 bool plan_is_device_ptr(const void* p) { return is_device_ptr(p); }
 }  // namespace lps

@@ -119,17 +119,18 @@ int reg_groups_of(int variant, int ncoil) {
   return 0;
 }
 
-void install(lps_plan* P, const TuneEntry& t) {
+int install(lps_plan* P, const TuneEntry& t) {
   const bool runtime = t.res.dc_variant == 1 || t.res.dc_variant == 2;
-  P->g.dc_generic = runtime;
-  P->g.dc_direct = t.res.dc_variant == 2;
-  P->g.dc_reg_groups = reg_groups_of(t.res.dc_variant, P->g.ncoil);
+  Geom g = P->g;
+  g.dc_generic = runtime;
+  g.dc_direct = t.res.dc_variant == 2;
+  g.dc_reg_groups = reg_groups_of(t.res.dc_variant, g.ncoil);
   if (runtime) {
-    P->g.py = t.py;
-    P->g.pz = t.pz;
+    g.py = t.py;
+    g.pz = t.pz;
   }
-  P->g.lrs_tpc = t.res.lrs_tiles;
-  P->graph_valid = false;
+  g.lrs_tpc = t.res.lrs_tiles;
+  return plan_set_shapes(P, g);
 }
 
 // Mean device time of `reps` launches of `fn` on the plan's stream (after one warm-up).
@@ -215,7 +216,7 @@ int lps_autotune(lps_plan* P, lps_tune_result* out) {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
-      install(P, it->second);
+      if ((rc = install(P, it->second))) return rc;
       if (out) {
         *out = it->second.res;
         out->cached = 1;
@@ -223,9 +224,15 @@ int lps_autotune(lps_plan* P, lps_tune_result* out) {
       return LPS_OK;
     }
   }
-  // scratch control block (never converged) and events
-  DevCtrl* ctrl = nullptr;
-  CK(cudaMalloc(&ctrl, sizeof(DevCtrl)));
+  // scratch control block (never converged), Gram partials and statistics (the plan's own belong to
+  // its state), and events
+  constexpr size_t ctrl_bytes = (sizeof(DevCtrl) + 255) / 256 * 256;
+  const size_t gram_bytes = (plan_gram_part_bytes(P) + 255) / 256 * 256;
+  unsigned char* scratch = nullptr;
+  CK(cudaMalloc(&scratch, ctrl_bytes + gram_bytes + (size_t)P->g.ntiles * 2 * sizeof(float)));
+  DevCtrl* ctrl = reinterpret_cast<DevCtrl*>(scratch);
+  float2* gram_part = reinterpret_cast<float2*>(scratch + ctrl_bytes);
+  float* lrs_part = reinterpret_cast<float*>(scratch + ctrl_bytes + gram_bytes);
   CK(cudaMemsetAsync(ctrl, 0, sizeof(DevCtrl), P->st));
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -243,7 +250,7 @@ int lps_autotune(lps_plan* P, lps_tune_result* out) {
     a.L = P->istage;    // scratch input and output: the plan's state is left alone
     a.S = nullptr;
     a.X = P->R;
-    a.gram_part = fp32 ? P->gram_part : nullptr;
+    a.gram_part = fp32 ? gram_part : nullptr;
     a.ctrl = ctrl;
     return time_launches(P, e0, e1, 5, [&] { return launch_dc(a, kDcUpdate, P->st); }, us);
   };
@@ -301,7 +308,7 @@ int lps_autotune(lps_plan* P, lps_tune_result* out) {
       l.L = P->istage;
       l.S = P->R;
       l.sup_prior = P->sup_prior;
-      l.lrs_part = P->lrs_part;
+      l.lrs_part = lrs_part;
       l.persist = P->persist;
       l.ctrl = ctrl;
       double us;
@@ -319,7 +326,7 @@ int lps_autotune(lps_plan* P, lps_tune_result* out) {
     best.res.radix_y[i] = (runtime && i < best.py.np) ? best.py.r[i] : 0;
     best.res.radix_z[i] = (runtime && i < best.pz.np) ? best.pz.r[i] : 0;
   }
-  install(P, best);
+  if ((rc = install(P, best))) goto done;
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune_cache[key] = best;
@@ -329,7 +336,7 @@ done:
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   cudaStreamSynchronize(P->st);
-  cudaFree(ctrl);
+  cudaFree(scratch);
   return rc;
 }
 
@@ -363,7 +370,8 @@ int lps_apply_tune(lps_plan* P, const lps_tune_result* t) {
     ARG(plan_of(t->radix_z, P->g.zn, e.pz), "radix_z does not factor the z transform length");
   }
   ARG(cudaStreamSynchronize(P->st) == cudaSuccess, "stream error");
-  install(P, e);
+  const int rc = install(P, e);
+  if (rc) return rc;
   if (dc_smem_bytes(P->g) > 227 * 1024) {
     set_err("the plane does not fit one CTA with this variant");
     return LPS_ERR_UNSUPPORTED;

@@ -125,6 +125,8 @@ int plan_build_graph(lps_plan* P);        // capture + instantiate the per-frame
 int plan_need_ready(lps_plan* P);         // coils, mask and data set
 int plan_upload_persist(lps_plan* P, bool with_v);
 int plan_frame_done(lps_plan* P);         // host bookkeeping after one frame of the graph ran
+int plan_set_shapes(lps_plan* P, const Geom& g);   // other launch shapes, the state's partials brought in line
+size_t plan_gram_part_bytes(const lps_plan* P);
 DcArgs plan_dc_args(lps_plan* P);
 bool plan_is_device_ptr(const void* p);
 
