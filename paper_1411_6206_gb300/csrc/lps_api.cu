@@ -194,11 +194,13 @@ int gram_part_capacity(const Geom& g) { return std::max(g.nx, gram_tc_parts(g));
 // Offset in the pinned control copy of the statistics that lps_data_consistency's kernel writes there.
 constexpr size_t kHostPart = (sizeof(DevCtrl) + 255) / 256 * 256;
 
-// Row tasks (where the plane has them), line positions and raster numbers of a mask.
-size_t line_table_bytes(const Geom& g) {
-  const size_t lines = (size_t)g.plane * sizeof(int);
-  return dc_rows_geometry(g) ? dc_row_task_bytes(g) + lines + (size_t)g.plane * sizeof(short) : lines;
+// Tables of a mask: row tasks and raster numbers (where the plane has them), then line positions. Their
+// places do not depend on the mask, so that a launch captured by the user stays right when another
+// mask is set; the positions come last and are copied as far as there are lines.
+size_t line_table_offset(const Geom& g) {
+  return dc_rows_geometry(g) ? dc_row_task_bytes(g) + (size_t)g.plane * sizeof(short) : 0;
 }
+size_t line_table_bytes(const Geom& g) { return line_table_offset(g) + (size_t)g.plane * sizeof(int); }
 
 size_t arena_size(const Geom& g, int max_iters) {
   auto r = [](size_t b) { return ((b + 255) / 256) * 256; };
@@ -207,7 +209,7 @@ size_t arena_size(const Geom& g, int max_iters) {
   s += 4 * r((size_t)g.nc * g.nc * sizeof(float2));      // W, V, float64 mode: Gram, refined V
   s += r((size_t)g.nc * g.nc * sizeof(double2)) + r((size_t)g.nc * sizeof(double));   // A, eigenvalues
   s += r((size_t)g.nxt * sizeof(float2)) + r((size_t)g.ny * sizeof(float2)) + r((size_t)g.nz * sizeof(float2));
-  s += r(line_table_bytes(g));                            // row tasks, line table, raster numbers
+  s += r(line_table_bytes(g));                            // row tasks, raster numbers, line table
   s += r((size_t)g.nx * 4 * sizeof(float)) + 2 * r((size_t)g.ntiles * 2 * sizeof(float));   // statistic partials
   s += 2 * r((size_t)g.nc * sizeof(double));
   s += 3 * r((size_t)(g.N / 32) * sizeof(uint32_t));   // support: prior, output, second output
@@ -893,8 +895,11 @@ int lps_plan_create(const lps_params* p, void* stream, lps_plan** out) {
   {
     unsigned char* t;
     if ((rc = aalloc(P, &t, line_table_bytes(g)))) return fail(rc);
-    if (dc_rows_geometry(g)) P->tasks = reinterpret_cast<RowTask*>(t);
-    P->lines = reinterpret_cast<int*>(t + (P->tasks ? dc_row_task_bytes(g) : 0));
+    if (dc_rows_geometry(g)) {
+      P->tasks = reinterpret_cast<RowTask*>(t);
+      P->raster = reinterpret_cast<unsigned short*>(t + dc_row_task_bytes(g));
+    }
+    P->lines = reinterpret_cast<int*>(t + line_table_offset(g));
   }
   if ((rc = aalloc(P, &P->hist, (size_t)p->max_iters + 2))) return fail(rc);
   if ((rc = aalloc(P, &P->gram_part, (size_t)gram_part_capacity(g) * g.nc * g.nc))) return fail(rc);
@@ -988,20 +993,18 @@ int lps_set_mask(lps_plan* P, const uint8_t* mask, int* nlines) {
   int slot;
   if ((rc = acquire_slot(P, &slot))) return rc;
   unsigned char* hs = P->h_lines_slots + (size_t)slot * line_table_bytes(P->g);
+  const size_t off = line_table_offset(P->g);
+  int* hl = reinterpret_cast<int*>(hs + off);
   if (P->tasks) {
-    const size_t tb = dc_row_task_bytes(P->g);
-    int* hl = reinterpret_cast<int*>(hs + tb);
-    dc_row_tasks(P->g, h, hs, hl, reinterpret_cast<unsigned short*>(hl + m));
-    P->raster = reinterpret_cast<unsigned short*>(P->lines + m);
-    CK(cudaMemcpyAsync(P->tasks, hs, tb + (size_t)m * (sizeof(int) + sizeof(short)), cudaMemcpyHostToDevice, P->st));
+    dc_row_tasks(P->g, h, hs, hl, reinterpret_cast<unsigned short*>(hs + dc_row_task_bytes(P->g)));
   } else {
-    int* hl = reinterpret_cast<int*>(hs);
     int k = 0;
     for (int a = 0; a < nz; ++a)
       for (int ky = 0; ky < ny; ++ky)
         if (h[(size_t)a * ny + ky]) hl[k++] = a * P->g.nyp + ky;
-    CK(cudaMemcpyAsync(P->lines, hl, (size_t)m * sizeof(int), cudaMemcpyHostToDevice, P->st));
   }
+  CK(cudaMemcpyAsync(P->tasks ? (void*)P->tasks : P->lines, hs, off + (size_t)m * sizeof(int), cudaMemcpyHostToDevice,
+                     P->st));
   P->nlines = m;
   P->hp.nlines = m;
   if ((rc = upload_persist(P, false, slot))) return rc;

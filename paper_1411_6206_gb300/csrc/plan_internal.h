@@ -61,8 +61,8 @@ struct lps_plan {
   float2* Lnew = nullptr;   // reprojection output of the precision modes
   float2 *tw_x = nullptr, *tw_y = nullptr, *tw_z = nullptr;
   int* lines = nullptr;
-  // row tasks of the mask (k_dc_rows), directly before the line table; nullptr where the plane has no
-  // such form. The lines are then kept in task order, and raster holds their numbers in the user's.
+  // row tasks of the mask (k_dc_rows), before the raster numbers and the line table; nullptr where the plane has
+  // no such form. The lines are then kept in task order, and raster holds their numbers in the user's.
   lps::RowTask* tasks = nullptr;
   unsigned short* raster = nullptr;
   float *dc_part = nullptr, *lrs_part = nullptr;
@@ -86,7 +86,7 @@ struct lps_plan {
   static constexpr int kSlots = 8;
   DevCtrl* h_ctrl = nullptr;
   DevPersist* h_persist_slots = nullptr;   // [kSlots]
-  unsigned char* h_lines_slots = nullptr;  // [kSlots] row tasks, line table, raster numbers
+  unsigned char* h_lines_slots = nullptr;  // [kSlots] row tasks, raster numbers, line table
   cudaEvent_t slot_done[kSlots] = {};
   bool slot_pending[kSlots] = {};
   int slot_next = 0;
