@@ -91,7 +91,8 @@ size_t dc_persist_smem(const Geom& g) {
 cudaError_t launch_dc_persist(const DcArgs* table, const int* start, int nm, int* counter, size_t smem,
                               cudaStream_t st) {
   // the kernel's static shared memory (its argument copy) counts against the same 227 KB
-  cudaError_t e = cudaFuncSetAttribute(k_dc_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_dc_persist), smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);

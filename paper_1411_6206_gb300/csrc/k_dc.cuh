@@ -329,14 +329,10 @@ __host__ __device__ constexpr int dc_ept_of(int plane) {
 
 template <int EPT, int MODE, bool STAGE, bool HALF>
 static cudaError_t launch_dc_t(const DcArgs& a, size_t smem, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_dc<EPT, MODE, STAGE, HALF>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)227 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  cudaError_t e = launch_pdl(k_dc<EPT, MODE, STAGE, HALF>, dim3(a.g.nx), dim3(kThreads), smem,
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_dc<EPT, MODE, STAGE, HALF>), 227 * 1024);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_dc<EPT, MODE, STAGE, HALF>, dim3(a.g.nx), dim3(kThreads), smem,
                              st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -451,13 +451,9 @@ static cudaError_t launch_fixed(const DcArgs& a, cudaStream_t st) {
   using Lay = DcFixedLayout<NY, NZ, NCG, NT>;
   constexpr size_t smem = Lay::bytes();
   static_assert(smem <= 227 * 1024, "plane does not fit shared memory");
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_dc_fixed<NY, NZ, NCG, NT, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_dc_fixed<NY, NZ, NCG, NT, MODE>), smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.g.nx);
   cfg.blockDim = dim3(NCG * NT);
@@ -472,7 +468,7 @@ static cudaError_t launch_fixed(const DcArgs& a, cudaStream_t st) {
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_dc_fixed<NY, NZ, NCG, NT, MODE>, a);
+  e = cudaLaunchKernelEx(&cfg, k_dc_fixed<NY, NZ, NCG, NT, MODE>, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -385,13 +385,9 @@ template <int G, bool FFTZ, bool ONE, bool ACCS, bool HALF, bool DH = false>
 cudaError_t launch_reg(const DcArgs& a, cudaStream_t st) {
   constexpr size_t smem = RegLayout<G, ACCS>::bytes();
   static_assert(smem <= 227 * 1024, "shared memory");
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_dc_reg<G, FFTZ, ONE, ACCS, HALF, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_dc_reg<G, FFTZ, ONE, ACCS, HALF, DH>), smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.g.nx);
   cfg.blockDim = dim3(G * kGT);
@@ -406,7 +402,7 @@ cudaError_t launch_reg(const DcArgs& a, cudaStream_t st) {
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_dc_reg<G, FFTZ, ONE, ACCS, HALF, DH>, a);
+  e = cudaLaunchKernelEx(&cfg, k_dc_reg<G, FFTZ, ONE, ACCS, HALF, DH>, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

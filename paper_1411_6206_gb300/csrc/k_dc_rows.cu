@@ -35,14 +35,10 @@ namespace {
 
 template <int MODE>
 cudaError_t launch_any(const DcArgs& a, const RowLaunch& q, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_dc_rows<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)227 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  return rows_launch(reinterpret_cast<const void*>(k_dc_rows<MODE>), a, q, st);
+  static SmemLimit limit;
+  const void* kernel = reinterpret_cast<const void*>(k_dc_rows<MODE>);
+  const cudaError_t e = limit.raise(kernel, 227 * 1024);
+  return e != cudaSuccess ? e : rows_launch(kernel, a, q, st);
 }
 
 bool rows_fixed(const Geom& g) { return rows_fixed_ny(g.ny) && rows_fixed_nz(g.nz); }

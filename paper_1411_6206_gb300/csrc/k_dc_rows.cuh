@@ -612,14 +612,10 @@ __global__ void __launch_bounds__(row_threads(NY), row_fit(NY, NZ, false, false,
 
 template <int MODE, int NY, int NZ>
 cudaError_t launch_rows_fixed_mode(const DcArgs& a, const RowLaunch& q, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_dc_rows_fixed<MODE, NY, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)227 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  return rows_launch(reinterpret_cast<const void*>(k_dc_rows_fixed<MODE, NY, NZ>), a, q, st);
+  static SmemLimit limit;
+  const void* kernel = reinterpret_cast<const void*>(k_dc_rows_fixed<MODE, NY, NZ>);
+  const cudaError_t e = limit.raise(kernel, 227 * 1024);
+  return e != cudaSuccess ? e : rows_launch(kernel, a, q, st);
 }
 
 template <int NY, int NZ>

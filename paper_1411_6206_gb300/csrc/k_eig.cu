@@ -786,13 +786,9 @@ __global__ void __launch_bounds__(kEigThreads, 1) k_eig(const EigArgs a) {
 template <int NCT, int CL>
 static cudaError_t launch_eig_c(const EigArgs& a, cudaStream_t st) {
   const size_t smem = sizeof(EigShared);
-  static bool attr_set = false;
-  if (smem > 48 * 1024 && !attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_eig<NCT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  cudaError_t e;
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_eig<NCT, CL>), smem);
+  if (e != cudaSuccess) return e;
   if constexpr (CL == 1) {
     e = launch_pdl(k_eig<NCT, 1>, dim3(1), dim3(kEigThreads), smem, st, a);
   } else {

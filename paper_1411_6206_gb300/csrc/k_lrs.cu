@@ -359,11 +359,10 @@ int lrs_blocks(const Geom& g) { return (g.ntiles + lrs_tpc(g) - 1) / lrs_tpc(g);
 template <int J, bool Z3>
 static cudaError_t launch_lrs_j(const LrsArgs& a, cudaStream_t st) {
   const size_t smem = lrs_smem(a.g);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_lrs<J, Z3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  cudaError_t e = launch_pdl(k_lrs<J, Z3>, dim3(lrs_blocks(a.g)), dim3(lrs_threads(a.g)), smem, st, a);
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_lrs<J, Z3>), smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_lrs<J, Z3>, dim3(lrs_blocks(a.g)), dim3(lrs_threads(a.g)), smem, st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -214,15 +214,11 @@ cudaError_t launch_gram_f32(const float2* X, const float2* S, const Geom& g, flo
   const long long nr = g.N / g.nc;
   if (nparts <= 0) return cudaErrorInvalidValue;
   const size_t smem = std::max((size_t)g.nc * (kGramRows | 1), (size_t)16 * kGramThreads) * sizeof(float2);
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_gram_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(kMaxNc * (kGramRows | 1) * sizeof(float2)));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const cudaError_t e = launch_pdl(k_gram_f32, dim3(nparts), dim3(kGramThreads), smem, st, X, S, g.nc, nr,
-                                   (nr + nparts - 1) / nparts, gram_part);
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_gram_f32), smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_gram_f32, dim3(nparts), dim3(kGramThreads), smem, st, X, S, g.nc, nr,
+                 (nr + nparts - 1) / nparts, gram_part);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -238,15 +234,11 @@ static cudaError_t launch_reproj_ng(const float2* X, const float2* S, const floa
   const long long nr = g.N / g.nc;
   constexpr int P = 4 * reproj_pg(NG), NC = 8 * NG;
   constexpr size_t smem = NC * NC * sizeof(float4) + (size_t)NC * P * sizeof(float2);
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_reproj_f32<NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const cudaError_t e = launch_pdl(k_reproj_f32<NG>, dim3((unsigned)((nr + P - 1) / P)), dim3(NG * reproj_pg(NG)), smem,
-                                   st, X, S, W, L, g.nc, nr);
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_reproj_f32<NG>), smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_reproj_f32<NG>, dim3((unsigned)((nr + P - 1) / P)), dim3(NG * reproj_pg(NG)), smem, st, X, S, W, L,
+                 g.nc, nr);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -470,13 +470,10 @@ size_t reproj_tc_smem(const Geom& g, int precision) {
 template <class Op>
 static cudaError_t launch_gram_op(const GramTcArgs& a, int precision, cudaStream_t st) {
   const size_t smem = gram_tc_smem(precision);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_tc<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  cudaError_t e = launch_pdl(k_gram_tc<Op>, dim3(gram_tc_parts(a.g)), dim3(kGramTcThreads), smem, st, a);
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_gram_tc<Op>), smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_gram_tc<Op>, dim3(gram_tc_parts(a.g)), dim3(kGramTcThreads), smem, st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -490,16 +487,13 @@ cudaError_t launch_gram_tc(const GramTcArgs& a, int precision, cudaStream_t st) 
 template <class Op>
 static cudaError_t launch_reproj_op(const ReprojTcArgs& a, int precision, cudaStream_t st) {
   const size_t smem = reproj_tc_smem(a.g, precision);
-  static size_t set_for = 0;
-  if (set_for < smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_reproj_tc<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    set_for = smem;
-  }
+  static SmemLimit limit;
+  cudaError_t e = limit.raise(reinterpret_cast<const void*>(k_reproj_tc<Op>), smem);
+  if (e != cudaSuccess) return e;
   const long long nr = (long long)a.g.nx * a.g.ny;
   const int ntiles = (int)((nr + kTcTile - 1) / kTcTile);
   const int grid = ntiles < 3 * 152 ? ntiles : 3 * 152;   // about what shares the SMs; more go on from tile to tile
-  cudaError_t e = launch_pdl(k_reproj_tc<Op>, dim3(grid), dim3(kTcThreads), smem, st, a);
+  e = launch_pdl(k_reproj_tc<Op>, dim3(grid), dim3(kTcThreads), smem, st, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -82,10 +82,9 @@ cudaError_t launch_xfft(const XfftArgs& a, cudaStream_t st) {
   if (er == cudaErrorNotSupported) er = launch_xfft_rows<3>(a, st);
   if (er != cudaErrorNotSupported) return er;
   const size_t smem = xfft_smem_bytes(a.g);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_xfft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static SmemLimit limit;
+  er = limit.raise(reinterpret_cast<const void*>(k_xfft), smem);
+  if (er != cudaSuccess) return er;
   const int cap = a.g.mpad;
   dim3 grid((cap + kLines - 1) / kLines, a.g.ncoil);
   k_xfft<<<grid, kThreads, smem, st>>>(a);

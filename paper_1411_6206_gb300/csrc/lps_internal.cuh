@@ -8,6 +8,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "smem_limit.h"
+
 namespace lps {
 
 constexpr int kThreads = 256;          // threads per CTA of the per-plane and per-tile kernels
