@@ -108,6 +108,14 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+// Start of both kernels, by one warp of a CTA. The successor is released behind the allocation and by
+// the warp that made it: a CTA counts as having released with the first of its threads that does. Were that
+// another warp, CTAs of a later launch of these kernels could take the tensor memory that this CTA still waits
+// for, and then wait for this launch to end.
+__device__ __forceinline__ void alloc_and_release(uint32_t* slot) {
+  tmem_alloc(slot);
+  pdl_trigger();
+}
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kTmemCols) : "memory");
 }
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(kGramTcThreads) k_gram_tc(const GramTcArgs a) 
   const int ntiles = (int)((nr + kTcTile - 1) / kTcTile);
   int* errp = a.ctrl ? &a.ctrl->err : nullptr;
 
-  if (warp == 0) tmem_alloc(tslot);
+  if (warp == 0) alloc_and_release(tslot);
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -196,7 +204,6 @@ __global__ void __launch_bounds__(kGramTcThreads) k_gram_tc(const GramTcArgs a) 
     *reinterpret_cast<uint4*>(stage[0] + i) = make_uint4(0u, 0u, 0u, 0u);
     *reinterpret_cast<uint4*>(stage[1] + i) = make_uint4(0u, 0u, 0u, 0u);
   }
-  pdl_trigger();
   pdl_wait();   // X and S come from the preceding kernels
   fence_proxy_async();
   tc_fence_before();
@@ -337,12 +344,11 @@ __global__ void __launch_bounds__(kTcThreads) k_reproj_tc(const ReprojTcArgs a) 
   const int ntiles = (int)((nr + kTcTile - 1) / kTcTile);
   int* errp = a.ctrl ? &a.ctrl->err : nullptr;
 
-  if (warp == 0) tmem_alloc(tslot);
+  if (warp == 0) alloc_and_release(tslot);
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     fence_mbar_init();
   }
-  pdl_trigger();
   pdl_wait();   // W, X and S come from the preceding kernels
   const int conv = a.ctrl ? a.ctrl->converged : 0;
   // the first tile's loads are on their way while B is built

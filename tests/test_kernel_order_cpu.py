@@ -1,6 +1,6 @@
 """Orders in the kernels' sources that no run can show to be missing (a race may never show): another
-CTA's shared memory is touched only behind a meeting of the cluster, and an operator call reads the maps
-and the samples only behind its dependency wait."""
+CTA's shared memory is touched only behind a meeting of the cluster, an operator call reads the maps and
+the samples only behind its dependency wait, and tensor memory is held before a successor may start."""
 import os
 import re
 
@@ -54,3 +54,15 @@ def test_operator_calls_wait_before_they_read_maps_or_samples(file, function, fi
     """Outside a frame (no control block) the call may directly follow the kernel that wrote them."""
     b = body(code(file), function)
     assert "if (!a.ctrl) pdl_wait();" in b[:b.index(first_read)]
+
+
+@pytest.mark.parametrize("function", ["k_gram_tc", "k_reproj_tc"])
+def test_tensor_memory_is_held_before_the_successor_is_released(function):
+    """A later launch must not take the tensor memory that a CTA of this one still waits for: the warp that
+    allocates is the one that releases, afterwards."""
+    src = code("k_tc.cu")
+    b = body(src, function)
+    assert "pdl_trigger()" not in b and "tmem_alloc(" not in b
+    assert "if (warp == 0) alloc_and_release(tslot);" in b[:b.index("pdl_wait()")]
+    r = body(src, "alloc_and_release")
+    assert r.index("tmem_alloc(") < r.index("pdl_trigger()")
