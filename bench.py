@@ -20,6 +20,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -123,9 +124,31 @@ class Clocks:
                 "reasons": reasons, "samples": len(rows)}
 
 
+def source_digest(path):
+    """sha256 of a kernel's source and of every file that it includes by name in quotes, and these in
+    turn (the transforms of a kernel are in headers of their own), each once, in order of their paths."""
+    seen, todo = {}, [os.path.normpath(path)]
+    while todo:
+        p = todo.pop()
+        if p in seen:
+            continue
+        with open(os.path.join(ROOT, p), "rb") as f:
+            seen[p] = f.read()
+        for name in re.findall(rb'^\s*#include "([^"]+)"', seen[p], re.M):
+            for d in (os.path.dirname(p), "include"):
+                q = os.path.normpath(os.path.join(d, name.decode()))
+                if os.path.exists(os.path.join(ROOT, q)):
+                    todo.append(q)
+                    break
+    h = hashlib.sha256()
+    for p in sorted(seen):
+        h.update(p.encode() + b"\0" + seen[p] + b"\0")
+    return h.hexdigest()
+
+
 def profiled_traffic(summary):
     """DRAM bytes per launch from a committed ncu summary under profiles/, or None when the
-    kernel's source has changed since the counters were taken (its sha256 differs)."""
+    kernel's source, or a header of it, has changed since the counters were taken."""
     try:
         kv = {}
         with open(os.path.join(ROOT, "profiles", summary)) as f:
@@ -133,9 +156,8 @@ def profiled_traffic(summary):
                 if ":" in line and not line[0].isspace():
                     k, v = line.split(":", 1)
                     kv[k.strip()] = v.strip()
-        with open(os.path.join(ROOT, kv["kernel_source"]), "rb") as f:
-            if hashlib.sha256(f.read()).hexdigest() != kv["source_sha256"]:
-                return None
+        if source_digest(kv["kernel_source"]) != kv["source_sha256"]:
+            return None
         return int(kv["dram_bytes_per_launch"])
     except (OSError, KeyError, ValueError):
         return None
