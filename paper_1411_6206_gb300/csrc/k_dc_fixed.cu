@@ -485,7 +485,7 @@ static cudaError_t launch_fixed_mode(const DcArgs& a, int mode, cudaStream_t st)
 // once or twice, and this kernel's is the shorter one (one step (4) call with its residual read back,
 // 32 x 32 x 8, one coil: 22.5 us against 24.3 us on factored rows; an iteration 15.7 against 16.2 us).
 bool dc_small_applies(const Geom& g) {
-  return g.dc_small && !g.dc_generic && g.cs == 1 && g.nx % kGramCluster == 0 && g.ny == 32 && g.nz == 8;
+  return !g.dc_generic && g.cs == 1 && g.nx % kGramCluster == 0 && g.ny == 32 && g.nz == 8;
 }
 
 // Returns cudaErrorNotSupported when no specialisation matches (the caller falls back to the

@@ -305,7 +305,6 @@ int validate(const lps_params* p, Geom* gout) {
   // 128 x 16 planes: the update runs on the register-transform kernel (four coil groups; their
   // sums in shared memory when there are more than four coils)
   if (g.ny == 128 && g.nz == 16) g.dc_reg_groups = g.ncoil > 4 ? 104 : 4;
-  g.dc_small = 1;
   // planes that factor: every mode of the data-consistency kernel on factored rows
   g.dc_rows = dc_rows_geometry(g) ? 1 : 0;
   if (dc_ept(g) < 0 || dc_smem_bytes(g) > 227 * 1024) {

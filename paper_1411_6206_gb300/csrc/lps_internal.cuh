@@ -88,7 +88,6 @@ struct Geom {
   int dc_direct;            // runtime-sized kernel reads coil maps from global memory (no staging)
   int lrs_tpc;              // 8x8 tiles per CTA of the sparse-step kernel (0: 32 / nc)
   int dc_reg_groups;        // register-transform DC kernel (128 x 16 planes): coil groups, 0 = off
-  int dc_small;             // the 32 x 8 plane's own kernel (k_dc_fixed)
   int dc_rows;              // factored-row kernel (k_dc_rows) where the plane has one
 };
 
