@@ -767,8 +767,8 @@ def run_batched(args):
     for name, pers in (("member_kernels", False), ("persistent", True)):
         B.data_consistency(Z, X, persistent=pers)
         step[name + "_ms"] = round(float(np.median([B.data_consistency(Z, X, persistent=pers) for _ in range(5)])), 3)
-    step["how"] = ("step (4) of every problem once: each member's tuned kernel (register-transform loop, "
-                   "compile-time or runtime-sized) as parallel graph branches, against one persistent launch "
+    step["how"] = ("step (4) of every problem once: each member's tuned kernel (factored rows "
+                   "or runtime-sized) as parallel graph branches, against one persistent launch "
                    "whose CTAs take (problem, plane) items from a counter and run the runtime-sized body; "
                    "median of 5, device time")
     res["dc_step_all_problems"] = step

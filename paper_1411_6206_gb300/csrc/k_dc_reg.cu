@@ -21,7 +21,7 @@
 // twiddles sit in two layouts and the line map rows 136 shorts apart for the same reason.
 // The prologue forms L_k = (X_{k-1} - S_{k-1}) W (steps 1-2) and the change statistic; the
 // epilogue sums the groups in a fixed order, writes X_k and the plane Gram (summed over
-// 4-CTA clusters through distributed shared memory), exactly as the staged-coil kernel does.
+// 4-CTA clusters through distributed shared memory).
 #include "lps_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(G * kGT, 1) k_dc_reg(const DcArgs a) {
     tjs[i] = a.tw_y[jb * sb];
   }
   for (int i = tid; i < kNZ * kLMS; i += NTH) lmap[i] = -1;
-  // sampled-line map: (kz, ky) -> line index (lines are kz * (ny + 1) + ky in raster order);
+  // sampled-line map: (kz, ky) -> line index (lines are kz * (ny + 1) + ky, in the plan's order);
   // the mask and its line table are set before any frame work
   const int m = a.persist->nlines;
   __syncthreads();   // the map was cleared above by other threads
@@ -410,8 +410,7 @@ cudaError_t launch_reg(const DcArgs& a, cudaStream_t st) {
 
 // The register-transform kernel covers the update form (steps 1-4 of an iteration, or
 // step 4 alone) of the 128 x 16 plane; the caller falls back to the other kernels on
-// cudaErrorNotSupported. It writes the same Gram partial count as the staged-coil kernel
-// (nx / 4, one per 4-plane cluster).
+// cudaErrorNotSupported. It writes nx / 4 Gram partials, one per 4-plane cluster.
 bool dc_reg_applies(const Geom& g) {
   return !g.dc_generic && g.cs == 1 && g.ny == kNY && g.nz == kNZ && g.nx % kRegCluster == 0 && g.dc_reg_groups > 0;
 }

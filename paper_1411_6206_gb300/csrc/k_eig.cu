@@ -363,8 +363,6 @@ __device__ __forceinline__ float2 gram_chunk(const float2* __restrict__ gram_par
   return make_float2(sx, sy);
 }
 
-// NCT: the column count fixed at compile time (its loops unroll and their loads pipeline);
-// 0 takes it from the geometry at run time.
 // CTA `rank`'s share of the Gram: ne entries, each summed over the partials in 512 / ne interleaved
 // chunks (a warp reads consecutive entries of a partial), the chunks added in order. Every partial
 // holds an exactly Hermitian matrix and every entry is summed in the same order, so the result is
@@ -405,6 +403,8 @@ __device__ __forceinline__ void gram_share(const EigArgs& a, EigShared& sh, int 
   cl.sync();
 }
 
+// NCT: the column count fixed at compile time (its loops unroll and their loads pipeline);
+// 0 takes it from the geometry at run time.
 // CL: cluster size. CTA r of a cluster sums the entries [r ne, (r + 1) ne) of the Gram, and stores them
 // in the first CTA's shared memory.
 template <int NCT, int CL>

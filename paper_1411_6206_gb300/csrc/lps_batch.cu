@@ -9,11 +9,12 @@
 // need not be rebuilt when members finish their sequences at different times.
 //
 // The autotuner times, on a plan's own resident data, the candidate launch shapes of the two
-// per-iteration kernels whose shape is a free choice: the data-consistency kernel (the
-// compile-time plane kernel where one exists, else the runtime-sized kernel with every
-// candidate ordering of FFT radix passes along y and z, with the coil planes staged in shared
-// memory or read from global memory) and the sparse-step kernel (8x8 tiles per CTA). The
-// fastest is installed in the plan; results are cached per geometry.
+// per-iteration kernels whose shape is a free choice: the data-consistency kernel (the plane's own
+// kernel or the factored-row kernel where there is one, both group counts of the register-transform
+// kernel on 128 x 16 planes, and the runtime-sized kernel with every candidate ordering of FFT radix
+// passes along y and z, with the coil planes staged in shared memory or read from global memory) and
+// the sparse-step kernel (8x8 tiles per CTA). The fastest is installed in the plan; results are cached
+// per geometry.
 #include "plan_internal.h"
 
 #include <algorithm>
@@ -352,7 +353,7 @@ int lps_apply_tune(lps_plan* P, const lps_tune_result* t) {
     Geom g = P->g;
     g.dc_generic = 0;
     g.dc_reg_groups = reg_groups_of(t->dc_variant, g.ncoil);
-    ARG(dc_has_fixed(g), "no compile-time kernel for this plane size");
+    ARG(dc_has_fixed(g), "no kernel under this number for this plane size");
     ARG(t->dc_variant == 0 || dc_reg_applies(g), "no register-transform kernel for this plane size");
   } else {
     auto plan_of = [&](const int* r, int n, FftPlan& f) -> bool {
